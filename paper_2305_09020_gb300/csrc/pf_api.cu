@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -244,11 +245,12 @@ struct Engine {
     unsigned long long tc_wait_ns_next = 0;          // the test hook's bound
     int nyp = 0;                      // row pitch of the y-transform intermediates (multiple of 4)
     int sms = 0;                      // multiprocessors of the device (persistent grid)
-    // TMA descriptors of the A operands, by (base, rows, K, pitch)
+    // TMA descriptors of the A operands (boxes of 128 rows) and of the outputs (32 rows), by (base,
+    // rows, K, pitch, box rows)
     struct AMap {
         const void *ptr;
         long long rows;
-        int K, pitch;
+        int K, pitch, box_rows;
         CUtensorMap map;
     };
     std::vector<AMap> amaps;
@@ -289,6 +291,27 @@ struct Engine {
         cur = 1 - c;
     }
 
+    // smallest and largest shift of each shift table, and whether every eigenvalue sum of a solve lies
+    // in [1e-15, 1e15] (the tensor-core transform's division then takes its branch-free form)
+    struct ShiftRange {
+        const T *sh;
+        double lo, hi;
+    };
+    std::vector<ShiftRange> shift_ranges;
+    void note_shifts(const T *sh, double lo, double hi) {
+        for (auto &r : shift_ranges)
+            if (r.sh == sh) { r.lo = lo; r.hi = hi; return; }
+        shift_ranges.push_back({sh, lo, hi});
+    }
+    bool div_safe(int bcset, const T *sh) const {
+        const std::vector<double> &a = hs.Lx, &b = hs.Ly[bcset];
+        for (auto &r : shift_ranges)
+            if (r.sh == sh)
+                return *std::min_element(a.begin(), a.end()) + *std::min_element(b.begin(), b.end()) + r.lo > 1e-14 &&
+                       *std::max_element(a.begin(), a.end()) + *std::max_element(b.begin(), b.end()) + r.hi < 1e14;
+        return false;
+    }
+
     template <typename U>
     U *mk(size_t n) {
         U *q = dalloc<U>(n);
@@ -325,7 +348,9 @@ struct Engine {
             for (int i = 0; i < ny; ++i)
                 for (int j = 0; j < ny; ++j) tmp[(size_t)i * ny + j] = s.Sy[b][(size_t)j * ny + i];
             SyT[b] = up(tmp);
-            Ly[b] = up(s.Ly[b]);
+            tmp = s.Ly[b];
+            tmp.resize((size_t)(ny + 63) / 64 * 64, 1.0);   // whole column tiles of the tensor-core transforms
+            Ly[b] = up(tmp);
         }
         liftV = up(s.liftV);
         if (s.patch) {
@@ -377,7 +402,9 @@ struct Engine {
                 const double beta = d3 ? 2.0 * M_PI * k / s.lz : 0.0;
                 v[pl] = c + beta * beta;
             }
-            return up(v);
+            T *q = up(v);
+            note_shifts(q, *std::min_element(v.begin(), v.end()), *std::max_element(v.begin(), v.end()));
+            return q;
         };
         shV = shifts(0.0);
         shP = shifts(0.0);
@@ -493,16 +520,18 @@ struct Engine {
     // right-hand sides and solutions keep pitch n_x; the y intermediates are padded to nyp)
     bool tc_possible() const { return nx % 4 == 0 && tc_encode() != nullptr; }
 
-    // column tiles of an N-column product: full tiles of BN = min(2 TC_MAXH, N rounded up to 16)
-    // columns and a last one that holds the rest (a multiple of 16)
+    // column tiles of an N-column product: full tiles of BN = min(2 TC_MAXH, N rounded up to 64)
+    // columns and a last one that holds the rest (multiples of 64: 32-column store rounds for both
+    // column halves; an MMA of N = 64 takes 48 cycles, of N = 48 44)
     static int tc_bn(int n, int *ntn, int *bnlast) {
-        const int npad = (n + 15) / 16 * 16;
+        const int npad = (n + 63) / 64 * 64;
         const int bn = std::min(2 * pf::TC_MAXH, npad);
         *ntn = (npad + bn - 1) / bn;
         *bnlast = npad - (*ntn - 1) * bn;
         return bn;
     }
 
+    // rows x K words at the given pitch, boxes of 32 columns x box_rows, 128-byte swizzle
     static void encode_2d(CUtensorMap *m, const void *ptr, long long rows, int K, int pitch, int box_rows) {
         cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
         cuuint64_t strides[1] = {(cuuint64_t)pitch * 4};
@@ -524,7 +553,7 @@ struct Engine {
         t.Npad = (t.ntn - 1) * t.BN + t.BNlast;
         t.Kpad = (n + pf::TC_KC - 1) / pf::TC_KC * pf::TC_KC;
         const size_t stage = (size_t)2 * pf::TC_BM * pf::TC_KC * 4 + (size_t)2 * t.BN * pf::TC_KC * 4;
-        const size_t fixed = 1024 + 512;   // alignment slack, barriers, TMEM slot, abort flag
+        const size_t fixed = 1024 + pf::TC_OUTBYTES + 512;   // alignment slack, store tiles, barriers, TMEM slot, abort flag
         t.stages = (int)std::min<size_t>(4, (size_t)(227 * 1024 - fixed) / stage);
         t.smem = t.stages * stage + fixed;
         t.tmem_cols = 512;                 // the ring of accumulation regions: one CTA per SM
@@ -547,20 +576,21 @@ struct Engine {
         tcb.push_back(t);
     }
 
-    const CUtensorMap &amap(const T *ptr, long long rows, int K, int pitch) {
+    CUtensorMap amap(const T *ptr, long long rows, int K, int pitch, int box_rows) {
         for (auto &a : amaps)
-            if (a.ptr == ptr && a.rows == rows && a.K == K && a.pitch == pitch) return a.map;
+            if (a.ptr == ptr && a.rows == rows && a.K == K && a.pitch == pitch && a.box_rows == box_rows) return a.map;
         AMap a;
-        a.ptr = ptr; a.rows = rows; a.K = K; a.pitch = pitch;
-        encode_2d(&a.map, ptr, rows, K, pitch, pf::TC_BM);
+        a.ptr = ptr; a.rows = rows; a.K = K; a.pitch = pitch; a.box_rows = box_rows;
+        encode_2d(&a.map, ptr, rows, K, pitch, box_rows);
         amaps.push_back(a);
-        return amaps.back().map;
+        return a.map;
     }
 
     // C = A B on the tensor cores (B one of the eigenbases registered by add_tc); A has `rows` rows
     // of K values at pitch lda; epilogue as pf::TcArgs
     void gemm_tc(const T *A, int lda, const T *B, T *C, long long rows, int R, int store, int ldc, int ldr,
-                 const T *lamN, const T *lamR, const T *cpl, int cpl_mod, T *C2 = nullptr, const T *face2 = nullptr) {
+                 const T *lamN, const T *lamR, const T *cpl, int cpl_mod, T *C2 = nullptr, const T *face2 = nullptr,
+                 bool div_ok = false) {
         const TcB *tb = nullptr;
         for (auto &t : tcb)
             if (t.key == B) tb = &t;
@@ -578,6 +608,7 @@ struct Engine {
         a.lamR = reinterpret_cast<const float *>(lamR);
         a.cpl = reinterpret_cast<const float *>(cpl);
         a.cpl_mod = cpl_mod;
+        a.div_ok = div_ok;
         a.C = reinterpret_cast<float *>(C);
         a.C2 = reinterpret_cast<float *>(C2);
         a.m2x = reinterpret_cast<const float *>(Mx);
@@ -587,11 +618,12 @@ struct Engine {
         a.wait_ns = tc_stall ? tc_wait_ns_next : tc_wait_ns;
         a.stall = tc_stall;
         tc_stall = 0;
-        const CUtensorMap &ma = amap(A, rows, tb->N, lda);
+        const CUtensorMap ma = amap(A, rows, tb->N, lda, pf::TC_BM);
+        const CUtensorMap mc = store == 0 ? amap(C, rows, tb->N, ldc, 32) : ma;
         if (sms == 0) sms = num_sms();
         const unsigned grid = (unsigned)std::min(a.ntiles, sms);
         prof->begin(PF_KC_GEMM, st);
-        pf::k_gemm_tc<<<grid, pf::TC_THREADS, tb->smem, st>>>(ma, tb->mh, tb->ml, a);
+        pf::k_gemm_tc<<<grid, pf::TC_THREADS, tb->smem, st>>>(ma, tb->mh, tb->ml, mc, a);
         check_launch();
         prof->end(st);
     }
@@ -607,7 +639,7 @@ struct Engine {
         // x: W1[p][x][y] (pitch nyp) = (rhs[p][y][:] Sx)^T
         gemm_tc(rhs, nx, Sx, W1, P * ny, ny, 1, 0, nyp, nullptr, nullptr, nullptr, 1);
         // y with the eigenvalue division: W2[p][x][:] = (W1[p][x][:] Sy) / (Ly + Lx + shift)
-        gemm_tc(W1, nyp, Sy[bcset], W2, P * nx, nx, 0, nyp, 0, Ly[bcset], Lx, sh, nz);
+        gemm_tc(W1, nyp, Sy[bcset], W2, P * nx, nx, 0, nyp, 0, Ly[bcset], Lx, sh, nz, nullptr, nullptr, div_safe(bcset, sh));
         // y^T: W1[p][y][x] (pitch nx) = (W2[p][x][:] Sy^T)^T
         gemm_tc(W2, nyp, SyT[bcset], W1, P * nx, nx, 1, 0, nx, nullptr, nullptr, nullptr, 1);
         // x^T: out[p][y][:] = W1[p][y][:] Sx^T (and the phi right-hand side -M psi (+ wall term))
@@ -1779,6 +1811,7 @@ int helm_impl(pf_handle *h, Engine<T> &E, int bcset, int mode, double lambda, co
     const double beta = E.d3 ? 2.0 * M_PI * mode / s.lz : 0.0;
     std::vector<T> sh(3 * E.nz, (T)(lambda + beta * beta));
     PF_CU(cudaMemcpyAsync(E.shTmp, sh.data(), sh.size() * sizeof(T), cudaMemcpyHostToDevice, E.st));
+    E.note_shifts(E.shTmp, (double)sh[0], (double)sh[0]);
     PF_CU(cudaMemcpyAsync(E.RHS, b.data(), b.size() * sizeof(T), cudaMemcpyHostToDevice, E.st));
     E.fdm(E.RHS, E.OUT, bcset, E.shTmp, np);
     std::vector<T> o((size_t)np * E.n2);
