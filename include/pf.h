@@ -52,7 +52,9 @@ extern "C" {
 #define PF_BC_NEUMANN   1
 #define PF_BC_PATCHES   2   /* wall only: electrodes on parts of the wall (eq. 21), see pf_vbc */
 
-#define PF_FP64  0   /* every kernel in double precision                                  */
+#define PF_FP64  0   /* every kernel in double precision; the eigenbasis GEMMs of planes of   */
+                     /* 28 to 480 nodes a side as exact products of 8-bit digits on the       */
+                     /* tensor cores, unless pf_set_variant pins a CUDA-core variant          */
 #define PF_MIXED 1   /* node-wise kernels and FFT in FP32, eigenbasis GEMMs in 3xTF32 on   */
                      /* the tensor cores (FP32 accumulation); set-up, the initial-potential */
                      /* fixed point and reductions in FP64                                  */
@@ -279,7 +281,9 @@ int pf_profile_read(pf_handle *h, double *ms, long long *launches);
  * the run (PF_GEMM_*), keep the fastest, then (unless a whole-plane variant won) whether the y transforms
  * run fused (one pass, eigenbasis in shared memory), then (3D) the z-transform tile of 4, 8, 16
  * or 32 pencils per block.  Each candidate is timed as the run executes its steady steps: graph
- * replays when the run has its own stream, eager launches on the legacy stream.  The run advances
+ * replays when the run has its own stream, eager launches on the legacy stream.  An FP64 run that
+ * is on the digit-product transforms times them as well and stays on them when they are fastest;
+ * choice then names the fastest CUDA-core variant, ms_per_step the run's time.  The run advances
  * by 16 (steps + 2) steps.  choice (nullable) receives gemm + 1000 * tile + 100000 * fused_y with
  * gemm a PF_GEMM_* code, tile the pencils per z-transform block (0: size heuristic, always 0 in
  * 2D) and fused_y 1 when the y pair runs fused; ms_per_step (nullable) the best time. */

@@ -26,6 +26,7 @@
 #include "../../include/pf.h"
 #include "pf_kernels.cuh"
 #include "pf_tc.cuh"
+#include "pf_oz.cuh"
 
 using pf::cplx;
 
@@ -254,6 +255,31 @@ struct Engine {
         CUtensorMap map;
     };
     std::vector<AMap> amaps;
+    // FP64 digit-product transforms (pf_oz.cuh): per B matrix its digits and column exponents; the digits
+    // and row exponents of the A operand; reciprocal eigenvalue sums per solve family
+    struct OzB {
+        const T *key;
+        __half *dig;      // [OZ_S][n][Kpad]
+        int *F;
+        int n, Kpad;
+    };
+    std::vector<OzB> ozb;
+    struct OzMap {
+        const void *ptr;
+        long long rows;
+        int Kpad, box;
+        CUtensorMap map;
+    };
+    std::vector<OzMap> ozmaps;
+    struct OzRcp {
+        int bcset;
+        const T *sh;
+        double *rcp;
+    };
+    std::vector<OzRcp> ozrcp;
+    __half *ozdig = nullptr;
+    int *ozE = nullptr;
+    bool use_oz = false;
     int simt_tile = 0;   // SIMT GEMM tile: 0 heuristic, 32 or 64 forced (autotuner)
     int tp_override = 0; // pencils per transform block: 0 heuristic, else forced (autotuner)
     // steady-state (BDF2) step captured once per history-slot parity; replayed by pf_step
@@ -503,7 +529,173 @@ struct Engine {
             for (auto &t : tcb) most = std::max(most, t.smem);
             raise_smem_limit((const void *)pf::k_gemm_tc, most);
         }
+        if (sizeof(T) == 8 && oz_pays()) {
+            use_oz = true;
+            auto tr = [](const std::vector<double> &m, int n) {
+                std::vector<double> t((size_t)n * n);
+                for (int i = 0; i < n; ++i)
+                    for (int j = 0; j < n; ++j) t[(size_t)i * n + j] = m[(size_t)j * n + i];
+                return t;
+            };
+            add_oz(Sx, tr(s.Sx, nx), nx);
+            add_oz(SxT, s.Sx, nx);
+            for (int b = 0; b < 4; ++b) {
+                add_oz(Sy[b], tr(s.Sy[b], ny), ny);
+                add_oz(SyT[b], s.Sy[b], ny);
+            }
+            raise_smem_limit((const void *)pf::k_gemm_oz, OZ_SMEM);
+            const long long most = (s.model == PF_MODEL_EQUILIBRIUM ? 1ll : d3 ? 3ll : 2ll) * nz;   // planes of a solve
+            ozdig = mk<__half>((size_t)pf::OZ_S * most * std::max((long long)ny * oz_kpad(nx), (long long)nx * oz_kpad(ny)));
+            ozE = mk<int>(most * std::max(nx, ny));
+            // reciprocals for the solves of the steady step (the others divide)
+            const int j = s.bdf == 2 ? 1 : 0;
+            add_rcp(PF_BCSET_V, shV);
+            if (s.precision == PF_FP64) {   // a mixed run's FP64 engine only finds the initial potential
+                add_rcp(PF_BCSET_NN, shPsi[j]);
+                add_rcp(PF_BCSET_NN, shPhi[j]);
+            }
+            if (s.precision == PF_FP64 && s.model != PF_MODEL_EQUILIBRIUM) {
+                add_rcp(PF_BCSET_P, shP);
+                add_rcp(PF_BCSET_U, shU[j]);
+            }
+        }
         PF_CU(cudaStreamSynchronize(st));
+    }
+
+    // ---- FP64 transforms by exact digit products on the tensor cores (pf_oz.cuh) -----------------
+    static constexpr size_t OZ_SMEM = 227 * 1024;
+    static int oz_kpad(int k) { return (k + pf::OZ_KC - 1) / pf::OZ_KC * pf::OZ_KC; }
+    // Eight launches a solve of about 5 us at least against the SIMT transforms' three or four: measured
+    // per 2D step, 24 x 13 nodes 0.277 / 0.271 ms (digits / SIMT), 30 x 16 0.279 / 0.289, 48 x 25 0.310 /
+    // 0.384, 240 x 121 0.571 / 1.276
+    bool oz_pays() const {
+        return std::max(nx, ny) >= 28 && nx <= pf::OZ_MAXK && ny <= pf::OZ_MAXK && tc_encode() != nullptr;
+    }
+    // digits and exponents of Bt's rows (Bt n x n row-major: B's columns)
+    void add_oz(const T *key, const std::vector<double> &Bt, int n) {
+        OzB t;
+        t.key = key;
+        t.n = n;
+        t.Kpad = oz_kpad(n);
+        std::vector<__half> dig((size_t)pf::OZ_S * n * t.Kpad, __float2half(0.f));
+        std::vector<int> F(n);
+        for (int r = 0; r < n; ++r) {
+            auto bits = [&](int k) {
+                unsigned long long u;
+                std::memcpy(&u, &Bt[(size_t)r * n + k], 8);
+                return u;
+            };
+            int em = 1;
+            for (int k = 0; k < n; ++k) em = std::max(em, (int)(bits(k) >> 52) & 0x7FF);
+            F[r] = em;
+            for (int k = 0; k < n; ++k) {
+                const unsigned long long u = pf::oz_fixed(bits(k), em);
+                for (int d = 0; d < pf::OZ_S; ++d) {
+                    const int v = d == 0 ? (int)(u >> 48) - 128 : (int)((u >> (8 * (6 - d))) & 0xFF) - 128;
+                    dig[((size_t)d * n + r) * t.Kpad + k] = __float2half((float)v);
+                }
+            }
+        }
+        t.dig = mk<__half>(dig.size());
+        t.F = mk<int>(n);
+        PF_CU(cudaMemcpyAsync(t.dig, dig.data(), dig.size() * sizeof(__half), cudaMemcpyHostToDevice, st));
+        PF_CU(cudaMemcpyAsync(t.F, F.data(), n * sizeof(int), cudaMemcpyHostToDevice, st));
+        PF_CU(cudaStreamSynchronize(st));
+        ozb.push_back(t);
+    }
+    void add_rcp(int bcset, const T *sh) {
+        const int modes = d3 ? nz / 2 + 1 : 1;
+        double *q = mk<double>((size_t)modes * nx * ny);
+        pf::k_oz_rcp<<<1024, 256, 0, st>>>(q, reinterpret_cast<const double *>(Ly[bcset]), reinterpret_cast<const double *>(Lx),
+                                           reinterpret_cast<const double *>(sh), modes, nz, nx, ny);
+        check_launch();
+        ozrcp.push_back({bcset, sh, q});
+    }
+    // digit planes [OZ_S][rows][Kpad], boxes of 32 x box x 7
+    CUtensorMap ozmap(const __half *ptr, long long rows, int Kpad, int box_rows) {
+        for (auto &m : ozmaps)
+            if (m.ptr == ptr && m.rows == rows && m.Kpad == Kpad && m.box == box_rows) return m.map;
+        OzMap m;
+        m.ptr = ptr; m.rows = rows; m.Kpad = Kpad; m.box = box_rows;
+        cuuint64_t dims[3] = {(cuuint64_t)Kpad, (cuuint64_t)rows, (cuuint64_t)pf::OZ_S};
+        cuuint64_t strides[2] = {(cuuint64_t)Kpad * 2, (cuuint64_t)Kpad * 2 * rows};
+        cuuint32_t box[3] = {(cuuint32_t)pf::OZ_KC, (cuuint32_t)box_rows, (cuuint32_t)pf::OZ_S};
+        cuuint32_t estr[3] = {1, 1, 1};
+        const CUresult r = tc_encode()(&m.map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half *>(ptr), dims, strides, box,
+                                       estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled"};
+        ozmaps.push_back(m);
+        return m.map;
+    }
+    void gemm_oz(const T *A, const T *B, T *C, long long rows, int R, int store, const T *lamN, const T *lamR,
+                 const T *cpl, const double *rcp, T *C2 = nullptr, const T *face2 = nullptr) {
+        const OzB *ob = nullptr;
+        for (auto &t : ozb)
+            if (t.key == B) ob = &t;
+        if (!ob) throw CudaError{cudaErrorInvalidValue, "digit-product transform without its eigenbasis"};
+        if (rows >= (1ll << 31) - pf::OZ_BM) throw CudaError{cudaErrorInvalidValue, "digit-product transform with 2^31 rows"};
+        if (sms == 0) sms = num_sms();
+        pf::OzArgs a{};
+        const int N = ob->n, mt = (int)((rows + pf::OZ_BM - 1) / pf::OZ_BM);
+        a.nst = ob->Kpad / pf::OZ_KC;
+        // column tiles: enough units for the chip, against the cycles of a unit: 56 MMAs a stage of
+        // 32 + N/4 cycles, about 2500 + 60 per column around them
+        double best = 0;
+        for (int nt = (N + 2 * pf::OZ_MAXH - 1) / (2 * pf::OZ_MAXH); nt <= (N + 15) / 16; ++nt) {
+            const int bn = ((N + nt - 1) / nt + 15) / 16 * 16, tiles = (N + bn - 1) / bn;
+            const double rounds = (double)(((long long)mt * tiles + sms - 1) / sms);
+            const double t = rounds * (a.nst * (56.0 * (36.0 + 0.25 * bn)) + 2500.0 + 60.0 * bn);
+            if (a.BN == 0 || t < 0.98 * best) { best = t; a.BN = bn; a.ntn = tiles; }
+        }
+        a.BNlast = ((N - (a.ntn - 1) * a.BN) + 15) / 16 * 16;
+        a.M = (int)rows; a.N = N; a.K = N;
+        a.tmem_cols = 512;
+        a.nr = std::min(pf::OZ_MAXR, 512 / a.BN) / 2 * 2;
+        const size_t stage = pf::OZ_ABYTES + (size_t)pf::OZ_S * a.BN * pf::OZ_KC * 2;
+        a.stages = (int)std::min<size_t>(4, (OZ_SMEM - pf::OZ_FIXED) / stage);
+        a.nunits = mt * a.ntn;
+        a.E = ozE; a.F = ob->F;
+        a.R = R; a.store = store; a.ldc = N; a.ldr = R;
+        a.lamN = reinterpret_cast<const double *>(lamN); a.lamR = reinterpret_cast<const double *>(lamR);
+        a.cpl = reinterpret_cast<const double *>(cpl); a.cpl_mod = nz;
+        a.rcp = rcp; a.rcp_modes = d3 ? nz / 2 + 1 : 1;
+        a.C = reinterpret_cast<double *>(C); a.C2 = reinterpret_cast<double *>(C2);
+        a.m2x = reinterpret_cast<const double *>(Mx); a.m2y = reinterpret_cast<const double *>(My);
+        a.face2 = reinterpret_cast<const double *>(face2);
+        a.active = active; a.amod = nz;
+        a.err = dev_err; a.wait_ns = tc_wait_ns;
+        const CUtensorMap ma = ozmap(ozdig, rows, ob->Kpad, pf::OZ_BM), mb = ozmap(ob->dig, N, ob->Kpad, a.BN);
+        const double *A64 = reinterpret_cast<const double *>(A);
+        prof->begin(PF_KC_GEMM, st);
+        const unsigned sg = (unsigned)((rows + 7) / 8);
+        auto split = [&](auto ni) {
+            pf::k_oz_split<decltype(ni)::value><<<sg, 256, 0, st>>>(A64, a.M, N, ob->Kpad, ozdig, ozE, R, active, nz);
+        };
+        switch ((ob->Kpad + 63) / 64) {
+            case 1: split(std::integral_constant<int, 1>{}); break;
+            case 2: split(std::integral_constant<int, 2>{}); break;
+            case 3: split(std::integral_constant<int, 3>{}); break;
+            case 4: split(std::integral_constant<int, 4>{}); break;
+            case 5: split(std::integral_constant<int, 5>{}); break;
+            case 6: split(std::integral_constant<int, 6>{}); break;
+            default: split(std::integral_constant<int, 8>{});
+        }
+        check_launch();
+        prof->end(st);
+        prof->begin(PF_KC_GEMM, st);
+        pf::k_gemm_oz<<<(unsigned)std::min(a.nunits, sms), pf::OZ_THREADS, a.stages * stage + pf::OZ_FIXED, st>>>(ma, mb, a);
+        check_launch();
+        prof->end(st);
+    }
+    void fdm_oz(const T *rhs, T *out, int bcset, const T *sh, long long P, T *minus_m_out, const T *face) {
+        const double *rcp = nullptr;
+        for (auto &r : ozrcp)
+            if (r.bcset == bcset && r.sh == sh) rcp = r.rcp;
+        gemm_oz(rhs, Sx, W1, P * ny, ny, 1, nullptr, nullptr, nullptr, nullptr);
+        gemm_oz(W1, Sy[bcset], W2, P * nx, nx, 0, Ly[bcset], Lx, sh, rcp);
+        gemm_oz(W2, SyT[bcset], W1, P * nx, nx, 1, nullptr, nullptr, nullptr, nullptr);
+        gemm_oz(W1, SxT, out, P * ny, ny, 0, nullptr, nullptr, nullptr, nullptr, minus_m_out, face);
     }
 
     // host TF32 rounding to nearest, ties away from zero (the rounding of cvt.rna.tf32.f32)
@@ -869,6 +1061,7 @@ struct Engine {
     bool tc_hybrid = false;
     void set_gemm(int code) {
         use_tc = code == 0 || code == 8;
+        use_oz = false;
         tc_hybrid = code == 8;
         fuse_plane = code == 1;
         cluster = code == 6 ? 4 : code == 7 ? 2 : 0;
@@ -888,6 +1081,10 @@ struct Engine {
         const long long P = nplanes;
         if (use_tc && !tcb.empty() && !(tc_hybrid && bcset == PF_BCSET_NN)) {
             fdm_tc(rhs, out, bcset, sh, P, minus_m_out, face);
+            return;
+        }
+        if (use_oz) {
+            fdm_oz(rhs, out, bcset, sh, P, minus_m_out, face);
             return;
         }
         if (cluster && cluster_fits(cluster)) {
@@ -1903,21 +2100,29 @@ void autotune_engine(Engine<T> &E, int steps, int total, cudaEvent_t e0, cudaEve
         PF_CU(cudaEventElapsedTime(&ms, e0, e1));
         return (double)ms / steps;
     };
+    // a run on the FP64 digit-product transforms times them first: they have no code of their own, and
+    // stay when no variant beats them
+    const bool digits = E.use_oz;
+    int taken = 0;
+    const double digits_ms = digits ? time_variant(taken) : INFINITY;
     // every variant this engine can run (PF_GEMM_* codes)
     std::vector<int> cands;
     for (int code : {0, 8, 32, 64, 2, 3, 4, 5, 1, 6, 7})
         if (E.gemm_available(code)) cands.push_back(code);
     int pick = cands[0];
     double best = INFINITY;
-    int taken = 0;
     for (int code : cands) {
         E.set_gemm(code);
         const double ms = time_variant(taken);
         if (ms < best) { best = ms; pick = code; }
     }
     E.set_gemm(pick);
+    if (digits_ms < best) {
+        E.use_oz = true;
+        best = digits_ms;
+    }
     // the fused y pair against the two separate y transforms (the whole-plane solves have no y pair)
-    if (!E.fuse_plane && !E.cluster) {
+    if (!E.fuse_plane && !E.cluster && !E.use_oz) {
         E.fuse_y = !E.fuse_y;
         const double ms = time_variant(taken);
         if (ms < best) best = ms;
@@ -2413,10 +2618,13 @@ extern "C" int pf_batch_autotune(pf_batch *b, int steps, double *ms_out) {
                 std::vector<int> cands;
                 for (int code : {0, 32, 64, 1, 6, 7})
                     if (E.gemm_available(code)) cands.push_back(code);
+                // the FP64 digit-product transforms (code -1 here) are timed too
+                if (E.use_oz) cands.push_back(-1);
                 int pick = cands[0];
                 int taken = 0;
                 for (int code : cands) {
-                    E.set_gemm(code);
+                    if (code < 0) E.use_oz = true;
+                    else E.set_gemm(code);
                     E.step(2);   // warm-up of this variant
                     PF_CU(cudaEventRecord(e0, E.st));
                     for (int s = 0; s < steps; ++s) E.step(2);
@@ -2427,7 +2635,8 @@ extern "C" int pf_batch_autotune(pf_batch *b, int steps, double *ms_out) {
                     PF_CU(cudaEventElapsedTime(&ms, e0, e1));
                     if (ms / steps < best) { best = ms / steps; pick = code; }
                 }
-                E.set_gemm(pick);
+                if (pick < 0) E.use_oz = true;
+                else E.set_gemm(pick);
                 for (; taken < total; ++taken) E.step(2);
             });
             if (ms_out) ms_out[gi] = best;

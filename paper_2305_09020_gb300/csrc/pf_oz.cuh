@@ -1,0 +1,458 @@
+// FP64 transform GEMM on the tensor cores (tcgen05 kind::f16, sm_103a): exact products of 8-bit digits.
+//
+// C[M x N] = A[M x K] * B[K x N] for the constant eigenbasis products of the Remark after Algorithm 2 in
+// double precision.  The FP64 pipe of the GB300 runs 2 FMA per SM and cycle (1.1 TFLOP/s measured), the
+// tensor cores 4096 FP16 products, and small integers multiply and add exactly there.  So each operand
+// is written in fixed point (the integer splitting of Ozaki, Ogita, Oishi and Rump for matrix units):
+//   row m of A:     a = X 2^(E_m - 1077),  X = rint(a 2^(1077 - E_m)), |X| < 2^55,
+//                   E_m the largest biased exponent of the row,
+//   column n of B:  b = Y 2^(F_n - 1077), the same (split once on the host),
+//   X = sum_s x_s 256^(6-s), seven balanced digits -128 <= x_s <= 128, stored as FP16 integers.
+// X Y summed over k is sum_d 256^(12-d) v_d with the level sums v_d = sum_{s+t=d} sum_k x_s y_t.  Levels
+// 0..6 (28 digit products) are kept: the first dropped level is 2^-56 of a product of two row maxima.
+// Within a stage of 32 k every level sum is an integer below 7 * 32 * 2^14 < 2^22, so the tensor core's
+// FP32 accumulation is exact.  The drain adds v_d, in units of 256^7, into 64-bit integers:
+//   acc += v_0 2^40 + v_1 2^32 + v_2 2^24 + v_3 2^16 + v_4 2^8 + v_5 + rint(v_6 / 256),
+// which also is exact but for v_6 and stays below 2^63 for K < 512.  The result is rounded to double once.
+// Against FMA chains, whose rounding grows with K, the error is smaller.
+//
+// A row with an infinity or NaN gives NaN results; other rows are not affected.  Subnormal entries keep
+// their bits; results are rounded to nearest, ties to even.
+#pragma once
+
+#include <cuda.h>
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "pf_tc.cuh"
+
+namespace pf {
+
+constexpr int OZ_S = 7;                       // digits per operand
+constexpr int OZ_KC = 32;                     // K per stage: 64-byte rows of FP16
+constexpr int OZ_BM = 128;                    // rows per unit = TMEM lanes
+constexpr int OZ_MAXH = 48;                   // accumulator columns per drain thread: BN <= 96
+constexpr int OZ_MAXK = 480;                  // K bound of the 64-bit sums (< 512)
+constexpr int OZ_MAXR = 16;                   // TMEM regions in the ring at most
+constexpr int OZ_EPI_WARPS = 8;
+constexpr int OZ_THREADS = 384;
+// the launch holds 384 x 168 = 64512 registers: 256 x 216 + 128 x 72 = 64512
+constexpr int OZ_REG_EPI = 216, OZ_REG_AUX = 72;
+static_assert(256 * OZ_REG_EPI + 128 * OZ_REG_AUX <= OZ_THREADS * 168, "the setmaxnreg split must fit the launch's registers");
+constexpr uint32_t OZ_ABYTES = OZ_S * OZ_BM * OZ_KC * 2;   // A digits of a stage
+constexpr int OZ_OUTP = 9;                    // row pitch (doubles) of a drain warp's 32 x 8 store block
+constexpr size_t OZ_OUTBYTES = (size_t)OZ_EPI_WARPS * 32 * OZ_OUTP * 8;
+constexpr size_t OZ_FIXED = 1024 + OZ_OUTBYTES + 512;      // alignment slack; store blocks; barriers, TMEM slot
+
+struct OzArgs {
+    int M, N, K;
+    int BN;                   // column tile (multiple of 16, <= 2 OZ_MAXH)
+    int ntn;                  // column tiles
+    int BNlast;               // width of the last one (multiple of 16)
+    int nst;                  // K stages
+    int nr;                   // TMEM regions (even, nr BN <= tmem_cols)
+    int stages;               // shared-memory stages
+    int tmem_cols;
+    int nunits;               // row tiles x column tiles
+    const int *E, *F;         // exponents of A's rows and B's columns
+    // epilogue: row m = p R + r; store 0: C[m ldc + n]; store 1: C[(p N + n) ldr + r]
+    int R, store, ldc, ldr;
+    const double *lamN, *lamR, *cpl;   // optional division by lamN[n] + lamR[r] + cpl[p % cpl_mod]
+    int cpl_mod;
+    const double *rcp;        // its reciprocals [mode][r][n], mode of plane p: 0 when rcp_modes == 1, else
+    int rcp_modes;            // that of the packed Fourier plane p % cpl_mod; null: divide
+    double *C;
+    double *C2;               // optional C2[m ldc + n] = -m2x[n] m2y[r] C (+ face2[p N + n] on r == 0)
+    const double *m2x, *m2y, *face2;
+    const int *active;        // ensembles: per-run flags (0 = frozen), run = p % amod; null otherwise
+    int amod;
+    int *err;
+    unsigned long long wait_ns;
+};
+
+// K-major, 64-byte swizzle, 8-row atoms of 512 bytes
+__device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFF);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
+    return d;
+}
+
+// instruction descriptor: D = F32, A = B = F16, both K-major, shape M x N
+__device__ __forceinline__ uint32_t idesc_f16(int M, int N) {
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t mbar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            dst),
+        "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(mbar)
+        : "memory");
+}
+
+// biased fixed point of a against the row exponent emax (>= a's): X + 128 (256^6 + .. + 1), so that byte s
+// from the top (16 bits for s = 0) is digit x_s + 128
+__host__ __device__ __forceinline__ unsigned long long oz_fixed(unsigned long long bits, int emax) {
+    const int e = (int)(bits >> 52) & 0x7FF;
+    unsigned long long m = bits & 0xFFFFFFFFFFFFFull;
+    if (e) m |= 1ull << 52;
+    int r = emax - (e ? e : 1);
+    if (r > 60) r = 60;
+    m = (((m << 3) >> r) + 1) >> 1;
+    const unsigned long long s = 0ull - (bits >> 63);
+    return ((m ^ s) - s) + 0x0080808080808080ull;
+}
+
+// value v 2^sc rounded to nearest even, by integer arithmetic (the FP64 pipe is the scarce unit here)
+__device__ __forceinline__ double oz_double(long long v, int sc) {
+    const unsigned long long sg = (unsigned long long)v & 0x8000000000000000ull;
+    unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)u);
+    u <<= lz & 63;
+    const unsigned long long m = u >> 11;
+    const unsigned int low = (unsigned int)u & 0x7FFu;
+    // half a unit plus the parity bit decides the carry: ties go to even
+    const unsigned long long up = (low + (unsigned int)(m & 1ull)) > 0x400u ? 1ull : 0ull;
+    int e = 1023 + 63 - lz + sc;             // biased exponent before rounding
+    double scale = 1.0;
+    const bool edge = e < 1 || e > 2045;     // subnormal or (almost) overflowing results
+    if (edge) {
+        if (v == 0) return 0.0;
+        // value = (normal number near 1) 2^(e - 1023), scaled by powers of two in range
+        const int t = min(max(e - 1023, -1100), 1100);
+        const double a = __longlong_as_double((long long)((((unsigned long long)1022 << 52) + m + up) | sg));
+        const int t1 = t / 2, t2 = t - t1;
+        scale = __longlong_as_double((long long)(1023 + t1) << 52);
+        return a * scale * __longlong_as_double((long long)(1023 + t2) << 52);
+    }
+    return v == 0 ? 0.0 : __longlong_as_double((long long)((((unsigned long long)(e - 1) << 52) + m + up) | sg));
+}
+
+#ifndef PF_OZ_HELPERS_ONLY
+// ---- digits of A: one warp per row ----------------------------------------------------------------
+// dig[d][m][Kpad] (FP16), E[m].  Bound by its 8 bytes read and 14 written per value, most of them in L2;
+// a pass of its own because inside the GEMM every column tile would split the rows again (measured there:
+// 7,000 issue slots per 128 x 32 stage against 3,100 cycles of MMAs).  NI = ceil(Kpad / 64) pairs a lane.
+template <int NI>
+__global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, int M, int K, int Kpad, __half *__restrict__ dig,
+                                                  int *__restrict__ E, int R, const int *__restrict__ active, int amod) {
+    const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (m >= M) return;
+    if (active && !active[(m / R) % amod]) return;   // a frozen run's rows: their products are not used
+    const double *row = A + (long long)m * K;
+    double x[NI][2];
+    unsigned int e = 0;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int k = 2 * (lane + 32 * i);
+        x[i][0] = k < K ? row[k] : 0.0;
+        x[i][1] = k + 1 < K ? row[k + 1] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+        e = max(e, max((unsigned int)__double2hiint(x[i][0]) & 0x7FF00000u, (unsigned int)__double2hiint(x[i][1]) & 0x7FF00000u));
+    const int em = max((int)(__reduce_max_sync(0xffffffffu, e) >> 20), 1);
+    if (lane == 0) E[m] = em;
+    const long long DS = (long long)M * Kpad / 2;     // words per digit plane
+    uint32_t *dst = reinterpret_cast<uint32_t *>(dig) + (long long)m * (Kpad / 2) + lane;
+    const __half2 bias = __half2half2(__ushort_as_half(0x6480));   // 1152
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        if (2 * (lane + 32 * i) >= Kpad) break;
+        const unsigned long long ua = oz_fixed((unsigned long long)__double_as_longlong(x[i][0]), em);
+        const unsigned long long ub = oz_fixed((unsigned long long)__double_as_longlong(x[i][1]), em);
+        const uint32_t al = (uint32_t)ua, ah = (uint32_t)(ua >> 32), bl = (uint32_t)ub, bh = (uint32_t)(ub >> 32);
+        auto put = [&](int d, uint32_t v) {   // v: two FP16 words 1024 + digit + 128
+            const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), bias);
+            dst[d * DS + 32 * i] = *reinterpret_cast<const uint32_t *>(&h);
+        };
+        put(0, __byte_perm(ah, bh, 0x7632) + 0x64006400u);
+        put(1, (__byte_perm(ah, bh, 0x0501) & 0x00FF00FFu) | 0x64006400u);
+        put(2, (__byte_perm(ah, bh, 0x0400) & 0x00FF00FFu) | 0x64006400u);
+        put(3, (__byte_perm(al, bl, 0x0703) & 0x00FF00FFu) | 0x64006400u);
+        put(4, (__byte_perm(al, bl, 0x0602) & 0x00FF00FFu) | 0x64006400u);
+        put(5, (__byte_perm(al, bl, 0x0501) & 0x00FF00FFu) | 0x64006400u);
+        put(6, (__byte_perm(al, bl, 0x0400) & 0x00FF00FFu) | 0x64006400u);
+    }
+}
+
+// reciprocals of the eigenvalue sums of one solve family, [mode][r][n] (0 where a sum is 0)
+static __global__ void k_oz_rcp(double *__restrict__ out, const double *__restrict__ lamN, const double *__restrict__ lamR,
+                                const double *__restrict__ shift, int modes, int nz, int R, int N) {
+    const long long n = (long long)modes * R * N;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const int k = (int)(i / ((long long)R * N));
+        const int r = (int)(i / N - (long long)k * R), c = (int)(i % N);
+        const int p = modes == 1 ? 0 : k == 0 ? 0 : (k == nz / 2 ? 1 : 2 * k);   // a packed plane of mode k
+        const double d = lamN[c] + lamR[r] + shift[p];
+        out[i] = d != 0.0 ? 1.0 / d : 0.0;
+    }
+}
+
+__device__ __forceinline__ bool oz_frozen(const OzArgs &g, int mt) {
+    if (!g.active) return false;
+    const int p1 = (min((mt + 1) * OZ_BM, g.M) - 1) / g.R;
+    for (int p = mt * OZ_BM / g.R; p <= p1; ++p)
+        if (g.active[p % g.amod]) return false;
+    return true;
+}
+
+// ---- the GEMM: persistent, warp-specialised; a CTA walks units of 128 rows x BN columns -------------
+//   warp 8      TMA: per 32-wide K stage the digits of A (32 x 128 x 7) and of B (32 x BN x 7), one 3D box each
+//   warps 9-10  issue the MMAs level by level (6 first; each level of a stage into a tensor-memory region
+//               of its own from a ring), the levels in turn between the two warps
+//   warps 0-7   drain the regions into the 64-bit integers, then convert and store (the epilogues of k_gemm)
+// setmaxnreg moves registers from warps 8-11 to the drain warps.  Every mbarrier wait is bounded as in
+// pf_tc.cuh: on time-out the error word is set, copies and MMAs in flight finish (bounded), tensor memory
+// is freed and the kernel returns.
+static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_constant__ CUtensorMap tmA,
+                                                                  const __grid_constant__ CUtensorMap tmB, OzArgs g) {
+    extern __shared__ __align__(1024) unsigned char oz_raw[];
+    unsigned char *base = (unsigned char *)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
+    const int S = g.stages, BN = g.BN, NR = g.nr;
+    const uint32_t BSL = (uint32_t)BN * OZ_KC * 2;            // bytes of one digit of B
+    const uint32_t STAGE = OZ_ABYTES + OZ_S * BSL;
+    double *outb = (double *)(base + (size_t)S * STAGE);
+    uint64_t *bars = (uint64_t *)((unsigned char *)outb + OZ_OUTBYTES);
+    // barriers: full[4] (a stage's digits landed), empty[4] (both issuers' MMAs done with it), rfull[16] /
+    // rempty[16] (a region's MMAs done / drained), fin[2]
+    const uint32_t b_full = smem_u32(bars), b_empty = b_full + 32, b_rfull = b_empty + 32, b_rempty = b_rfull + 8 * OZ_MAXR,
+                   b_fin = b_rempty + 8 * OZ_MAXR;
+    uint32_t *tslot = (uint32_t *)(bars + 8 + 2 * OZ_MAXR + 2);
+    volatile int *abort_flag = (volatile int *)(tslot + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    if (tid == 0) {
+        for (int s = 0; s < 4; ++s) {
+            mbar_init(b_full + 8 * s, 1);
+            mbar_init(b_empty + 8 * s, 2);
+        }
+        for (int r = 0; r < OZ_MAXR; ++r) {
+            mbar_init(b_rfull + 8 * r, 1);
+            mbar_init(b_rempty + 8 * r, OZ_EPI_WARPS);
+        }
+        mbar_init(b_fin, 1);
+        mbar_init(b_fin + 8, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(g.tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tslot;
+    auto fail = [&]() {
+        if (!*abort_flag) atomicExch(g.err, TC_ERR_TIMEOUT);
+        *abort_flag = 1;
+    };
+    const int ntn = g.ntn, nst = g.nst;
+
+    if (warp >= OZ_EPI_WARPS) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(OZ_REG_AUX));
+        if (warp == OZ_EPI_WARPS) {
+            // ---- TMA producer -----------------------------------------------------------------------
+            if (lane == 0) {
+                int s = 0, issued = 0;
+                uint32_t ph = 0;
+                bool ok = true;
+                for (int u = blockIdx.x; u < g.nunits && ok; u += gridDim.x) {
+                    const int mt = u / ntn, nt = u - mt * ntn;
+                    if (oz_frozen(g, mt)) continue;
+                    for (int c = 0; c < nst; ++c) {
+                        if (!mbar_wait(b_empty + 8 * s, ph ^ 1u, abort_flag, g.wait_ns)) { fail(); ok = false; break; }
+                        const uint32_t sa = smem_u32(base + (size_t)s * STAGE);
+                        mbar_expect_tx(b_full + 8 * s, STAGE);
+                        tma_load_3d(sa, &tmA, c * OZ_KC, mt * OZ_BM, 0, b_full + 8 * s);
+                        tma_load_3d(sa + OZ_ABYTES, &tmB, c * OZ_KC, nt * BN, 0, b_full + 8 * s);
+                        ++issued;
+                        if (++s == S) { s = 0; ph ^= 1u; }
+                    }
+                }
+                // copies still in flight (only after an abort) finish before the CTA leaves
+                for (int q = issued - 1; q >= 0 && q >= issued - S; --q)
+                    mbar_wait(b_full + 8 * (q % S), (uint32_t)((q / S) & 1), nullptr, g.wait_ns);
+            }
+            __syncwarp();
+        } else if (warp <= OZ_EPI_WARPS + 2) {
+            // ---- MMA issuers: whole warps, one elected lane (see pf_tc.cuh); issuer w takes every other
+            // level of the sequence (seven a stage), so each starts at its own region and skips one -----
+            const int w = warp - (OZ_EPI_WARPS + 1);
+            const uint32_t id_full = idesc_f16(OZ_BM, BN), id_last = idesc_f16(OZ_BM, g.BNlast);
+            int s = 0, r = w, turn = 0;
+            uint32_t ph = 0, rph = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; u < g.nunits && ok; u += gridDim.x) {
+                const int mt = u / ntn, nt = u - mt * ntn;
+                if (oz_frozen(g, mt)) continue;
+                const uint32_t idesc = nt == ntn - 1 ? id_last : id_full;
+                for (int c = 0; c < nst && ok; ++c) {
+                    if (!mbar_wait_warp(b_full + 8 * s, ph, abort_flag, g.wait_ns)) { fail(); ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t sa = smem_u32(base + (size_t)s * STAGE);
+                    const uint64_t da = sdesc_sw64(sa), db = sdesc_sw64(sa + OZ_ABYTES);
+                    const bool two = g.K - c * OZ_KC > 16;   // the last stage may hold one 16-wide step only
+#pragma unroll
+                    for (int d = OZ_S - 1; d >= 0; --d) {
+                        if (turn == w) {
+                            if (!mbar_wait_warp(b_rempty + 8 * r, rph ^ 1u, abort_flag, g.wait_ns)) { fail(); ok = false; break; }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint32_t t = tmem + (uint32_t)(r * BN);
+                            if (elect_one()) {
+#pragma unroll
+                                for (int x = 0; x <= d; ++x) {
+                                    const uint64_t a = da + (uint64_t)(x * ((OZ_BM * OZ_KC * 2) >> 4));
+                                    const uint64_t b = db + (uint64_t)((d - x) * (int)(BSL >> 4));
+                                    mma_f16(t, a, b, idesc, x ? 1u : 0u);
+                                    if (two) mma_f16(t, a + 2, b + 2, idesc, 1u);   // the next 16 k: 32 bytes further
+                                }
+                                mma_commit(b_rfull + 8 * r);
+                            }
+                            __syncwarp();
+                            r += 2;
+                            if (r >= NR) { r -= NR; rph ^= 1u; }
+                        }
+                        turn ^= 1;
+                    }
+                    if (!ok) break;
+                    if (elect_one()) mma_commit(b_empty + 8 * s);
+                    __syncwarp();
+                    if (++s == S) { s = 0; ph ^= 1u; }
+                }
+            }
+            // every MMA issued finishes before the tensor memory is released (also after an abort)
+            __syncwarp();
+            if (elect_one()) mma_commit(b_fin + 8 * w);
+            mbar_wait(b_fin + 8 * w, 0u, nullptr, g.wait_ns);
+            __syncwarp();
+        }
+    } else {
+        // ---- drain, epilogue (warps 0-7) ------------------------------------------------------------------
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REG_EPI));
+        const int quarter = warp & 3, half = warp >> 2;
+        long long acc[OZ_MAXH];
+#pragma unroll
+        for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
+        int r = 0;
+        uint32_t rph = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < g.nunits && ok; u += gridDim.x) {
+            const int mt = u / ntn, nt = u - mt * ntn;
+            if (oz_frozen(g, mt)) continue;
+            const int hbn = (nt == ntn - 1 ? g.BNlast : BN) >> 1;   // columns per thread (a multiple of 8)
+            const uint32_t lane0 = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * hbn);
+            for (int c = 0; c < nst && ok; ++c) {
+#pragma unroll
+                for (int d = OZ_S - 1; d >= 0; --d) {
+                    if (!mbar_wait(b_rfull + 8 * r, rph, abort_flag, g.wait_ns)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t ta = lane0 + (uint32_t)(r * BN);
+#pragma unroll
+                    for (int j0 = 0; j0 < OZ_MAXH; j0 += 16) {
+                        if (j0 < hbn) {   // 16 columns (those past hbn are another half's, or none's: not used)
+                            float v[16];
+                            tmem_ld16(ta + (uint32_t)j0, v);
+                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                // v is an integer below 2^22: its bits after adding 1.5 2^23
+                                const int w = __float_as_int(v[j] + 12582912.f) - 0x4B400000;
+                                long long &a = acc[j0 + j];
+                                if (d == 6) a += (long long)((w + 128) >> 8);
+                                else a += (long long)w * (1ll << (8 * (5 - d)));
+                            }
+                        }
+                    }
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(b_rempty + 8 * r);
+                    if (++r == NR) { r = 0; rph ^= 1u; }
+                }
+            }
+            if (!ok) break;
+            // ---- epilogue: eight columns per round, the rest moved down (a small loop: code is fetched at
+            // about five cycles an instruction here) --------------------------------------------------
+            const int m0 = mt * OZ_BM + quarter * 32, m = m0 + lane, nb = nt * BN + half * hbn;
+            const int em = m < g.M ? g.E[m] : 1;
+            const int p = m < g.M ? m / g.R : 0, rr = m < g.M ? m - p * g.R : 0;
+            double *ob = outb + warp * (32 * OZ_OUTP);
+            double *cb = g.C + ((long long)p * g.N + nb) * g.ldr + rr;   // store 1
+            const int ncol = min(hbn, g.N - nb);
+#pragma unroll 1
+            for (int j0 = 0; j0 < ncol; j0 += 8) {
+                double v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {   // units 2^56 of X Y 2^(E + F - 2154)
+                    v[j] = oz_double(acc[j], em + (j0 + j < ncol ? g.F[nb + j0 + j] : 1) - 2154 + 56);
+                    if (em == 0x7FF) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+                }
+                if (g.store == 1) {             // lanes hold consecutive rows: coalesced as it is
+#pragma unroll
+                    for (int j = 0; j < 8; ++j, cb += g.ldr)
+                        if (m < g.M && j0 + j < ncol) *cb = v[j];
+                } else {                        // through shared memory: eight lanes per row segment of 64 bytes
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) ob[lane * OZ_OUTP + j] = v[j];
+                    __syncwarp();
+                    const int n = nb + j0 + (lane & 7);
+                    const bool in = j0 + (lane & 7) < ncol;
+#pragma unroll 2
+                    for (int i = 0; i < 8; ++i) {
+                        const int row = 4 * i + (lane >> 3), mm = m0 + row;
+                        const int pp = __shfl_sync(0xffffffffu, p, row), r2 = __shfl_sync(0xffffffffu, rr, row);
+                        if (mm < g.M && in) {
+                            double x = ob[row * OZ_OUTP + (lane & 7)];
+                            if (g.rcp) {
+                                const int pl = pp % g.cpl_mod;
+                                const int md = g.rcp_modes == 1 ? 0 : (pl == 1 ? g.cpl_mod / 2 : pl >> 1);
+                                x *= g.rcp[((long long)md * g.R + r2) * g.N + n];
+                            } else if (g.lamN) {
+                                const double dd = g.lamN[n] + g.lamR[r2] + g.cpl[pp % g.cpl_mod];
+                                x = (dd != 0.0) ? x / dd : 0.0;
+                            }
+                            g.C[(long long)mm * g.ldc + n] = x;
+                            if (g.C2) {
+                                double w2 = -g.m2x[n] * g.m2y[r2] * x;
+                                if (g.face2 && r2 == 0) w2 += g.face2[(long long)pp * g.N + n];
+                                g.C2[(long long)mm * g.ldc + n] = w2;
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j + 8 < OZ_MAXH; ++j) acc[j] = acc[j + 8];
+            }
+#pragma unroll
+            for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
+        }
+        if (!ok) fail();
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.tmem_cols) : "memory");
+    }
+}
+#endif  // PF_OZ_HELPERS_ONLY
+
+}  // namespace pf
