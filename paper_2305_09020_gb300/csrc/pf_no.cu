@@ -113,25 +113,31 @@ __global__ void __launch_bounds__(128, 1) k_dense_fwd_tc(const float *__restrict
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *slot;
-    if (tid == 0) {
+    if (warp == 0) {   // a whole warp with one elected lane: 45 cycles an MMA instead of 226 (pf_tc.cuh)
         // instruction descriptor: D = F32, A = B = BF16, both K-major, M = 128, N = 64
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NO_TC_BN >> 3) << 17) |
                                ((uint32_t)(128 >> 4) << 24);
-        const uint32_t a0 = pf::smem_u32(sA), bh0 = pf::smem_u32(sBh), bl0 = pf::smem_u32(sBl);
-        for (int s = 0; s < K / 16; ++s) {   // 16 BF16 = 32 bytes per K step
-            const uint32_t oa = (uint32_t)((s >> 2) * 128 * 128 + (s & 3) * 32);
-            const uint32_t ob = (uint32_t)((s >> 2) * NO_TC_BN * 128 + (s & 3) * 32);
-            const uint64_t da = pf::sdesc_sw128(a0 + oa);
-            uint32_t acc = s > 0 ? 1u : 0u;
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-                         "l"(da), "l"(pf::sdesc_sw128(bh0 + ob)), "r"(idesc), "r"(acc));
-            acc = 1u;
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-                         "l"(da), "l"(pf::sdesc_sw128(bl0 + ob)), "r"(idesc), "r"(acc));
+        const uint64_t da0 = pf::sdesc_sw128(pf::smem_u32(sA)), dh0 = pf::sdesc_sw128(pf::smem_u32(sBh)),
+                       dl0 = pf::sdesc_sw128(pf::smem_u32(sBl));
+        for (int s0 = 0; s0 < K / 16; s0 += 4) {   // one 64-wide atom: four K steps of 16 BF16 = 32 bytes
+            if (pf::elect_one()) {
+                const uint64_t oa = (uint64_t)((s0 >> 2) * 128 * 128 >> 4), ob = (uint64_t)((s0 >> 2) * NO_TC_BN * 128 >> 4);
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    const uint64_t da = da0 + oa + 2 * s;
+                    const uint32_t acc = s0 + s > 0 ? 1u : 0u;
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
+                                 "l"(da), "l"(dh0 + ob + 2 * s), "r"(idesc), "r"(acc));
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
+                                 "l"(da), "l"(dl0 + ob + 2 * s), "r"(idesc), "r"(1u));
+                }
+            }
+            __syncwarp();
         }
-        pf::mma_commit(pf::smem_u32(mbar));
+        if (pf::elect_one()) pf::mma_commit(pf::smem_u32(mbar));
+        __syncwarp();
     }
     bool ok = pf::mbar_wait(pf::smem_u32(mbar), 0u, nullptr, 1000000000ull);
     if (!ok) {   // record the time-out, give the MMAs one more bounded wait before the memory goes
@@ -171,41 +177,99 @@ __global__ void k_transpose_bf16(const __nv_bfloat16 *__restrict__ W, __nv_bfloa
         if (n0 + i < N && k0 + threadIdx.x < K) Wt[(size_t)(n0 + i) * K + k0 + threadIdx.x] = t[threadIdx.x][i];
 }
 
-// dZ = dY (1 - Y^2) in place on dY
-__global__ void k_tanh_back(const float *__restrict__ Y, float *__restrict__ dY, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dY[i] *= 1.f - Y[i] * Y[i];
-}
-
-// dX[r][k] = sum_n dZ[r][n] W[k][n]: one warp per (r, k)
-__global__ void k_dense_bwd_x(const float *__restrict__ dZ, const __nv_bfloat16 *__restrict__ W,
-                              float *__restrict__ dX, int B, int K, int N) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= B * K) return;
-    const int r = warp / K, k = warp % K;
-    float s = 0.f;
-    for (int n = lane; n < N; n += 32) s += dZ[(long long)r * N + n] * __bfloat162float(W[(long long)k * N + n]);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) dX[(long long)r * K + k] = s;
-}
-
-// dW[k][n] = sum_r Xin[r][k] dZ[r][n] ; db[n] = sum_r dZ[r][n]
-__global__ void k_dense_bwd_w(const float *__restrict__ X, const float *__restrict__ dZ, float *__restrict__ dW,
-                              float *__restrict__ db, int B, int K, int N, const float *__restrict__ mean,
-                              const float *__restrict__ istd) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = blockIdx.y;
-    if (n >= N) return;
-    float s = 0.f, sb = 0.f;
-    for (int r = 0; r < B; ++r) {
-        float x = X[(long long)r * K + k];
-        if (mean) x = (x - mean[k]) * istd[k];
-        const float d = dZ[(long long)r * N + n];
-        s += x * d;
-        sb += d;
+// dZ_in[r][k] = (1 - Y^2) sum_n dZ[r][n] W[k][n]: a warp takes 4 samples x 4 inputs, its lanes the terms
+// n = lane (mod 32), each with its sixteen sums in registers; the lanes' sums are added at the end.
+// Four loads of each operand serve sixteen products (a warp per output read both operands from L2 once
+// per output, 1.2 GB a batch of the 384 -> 8192 layer); four steps of n are in flight.
+constexpr int BX_T = 4;
+__global__ void __launch_bounds__(256) k_dense_bwd_x(const float *__restrict__ dZ, const __nv_bfloat16 *__restrict__ W,
+                                                     const float *__restrict__ Y, float *__restrict__ dX, int B, int K, int N) {
+    const int lane = threadIdx.x & 31, warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int nk = (K + BX_T - 1) / BX_T, r0 = warp / nk * BX_T, k0 = warp % nk * BX_T;
+    if (r0 >= B) return;
+    const float *dp[BX_T];
+    const __nv_bfloat16 *wp[BX_T];
+#pragma unroll
+    for (int i = 0; i < BX_T; ++i) {   // rows past the end repeat the last one; their sums are not stored
+        dp[i] = dZ + (long long)min(r0 + i, B - 1) * N;
+        wp[i] = W + (long long)min(k0 + i, K - 1) * N;
     }
-    dW[(long long)k * N + n] = s;
-    if (k == 0) db[n] = sb;
+    float s[BX_T][BX_T] = {};
+#pragma unroll 4
+    for (int n = lane; n < N; n += 32) {
+        float d[BX_T], w[BX_T];
+#pragma unroll
+        for (int i = 0; i < BX_T; ++i) {
+            d[i] = dp[i][n];
+            w[i] = __bfloat162float(wp[i][n]);
+        }
+#pragma unroll
+        for (int i = 0; i < BX_T; ++i)
+#pragma unroll
+            for (int j = 0; j < BX_T; ++j) s[i][j] += d[i] * w[j];
+    }
+#pragma unroll
+    for (int i = 0; i < BX_T; ++i)
+#pragma unroll
+        for (int j = 0; j < BX_T; ++j) {
+            float v = s[i][j];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0 && r0 + i < B && k0 + j < K) {
+                const long long q = (long long)(r0 + i) * K + k0 + j;
+                const float y = Y[q];
+                dX[q] = v * (1.f - y * y);
+            }
+        }
+}
+
+// dW[k][n] = sum_r Xin[r][k] dZ[r][n] ; db[n] = sum_r dZ[r][n]: a thread takes output column n of 32 inputs
+// k, so dZ is read once per 32 rows of dW (a thread per element read it once per row: 0.8 GB a batch of the
+// 384 -> 8192 layer); the sums run over r in order
+constexpr int BW_K = 32, BW_R = 64;
+__global__ void __launch_bounds__(128) k_dense_bwd_w(const float *__restrict__ X, const float *__restrict__ dZ,
+                                                     float *__restrict__ dW, float *__restrict__ db, int B, int K, int N,
+                                                     const float *__restrict__ mean, const float *__restrict__ istd) {
+    __shared__ __align__(16) float sX[BW_R][BW_K];
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, k0 = blockIdx.y * BW_K;
+    float acc[BW_K] = {}, sb = 0.f;
+    for (int r0 = 0; r0 < B; r0 += BW_R) {
+        const int nr = min(BW_R, B - r0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < BW_R * BW_K; i += blockDim.x) {
+            const int r = i / BW_K, k = k0 + i % BW_K;
+            float x = 0.f;
+            if (r < nr && k < K) {
+                x = X[(long long)(r0 + r) * K + k];
+                if (mean) x = (x - mean[k]) * istd[k];
+            }
+            sX[r][i % BW_K] = x;
+        }
+        __syncthreads();
+        if (n < N)
+            for (int rb = 0; rb < nr; rb += 8) {
+                float d[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) d[i] = rb + i < nr ? dZ[(long long)(r0 + rb + i) * N + n] : 0.f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (rb + i >= nr) break;
+                    sb += d[i];
+#pragma unroll
+                    for (int k = 0; k < BW_K; k += 4) {
+                        const float4 x = *reinterpret_cast<const float4 *>(&sX[rb + i][k]);
+                        acc[k] += x.x * d[i];
+                        acc[k + 1] += x.y * d[i];
+                        acc[k + 2] += x.z * d[i];
+                        acc[k + 3] += x.w * d[i];
+                    }
+                }
+            }
+    }
+    if (n >= N) return;
+#pragma unroll
+    for (int k = 0; k < BW_K; ++k)
+        if (k0 + k < K) dW[(long long)(k0 + k) * N + n] = acc[k];
+    if (k0 == 0) db[n] = sb;
 }
 
 // nodes[r][q] = sum_{c<4} w[q][c] grid[r][idx[q][c]]
@@ -219,15 +283,17 @@ __global__ void k_resample(const float *__restrict__ G, const int *__restrict__ 
     out[(long long)r * nq + q] = s;
 }
 
-// transpose: dG[r][i] = sum over (q, c) with idx[q][c] = i of w[q][c] dN[r][q]  (CSR by grid point)
+// transpose, and the output layer's tanh': dZ[r][i] = (1 - Y^2) sum over (q, c) with idx[q][c] = i of
+// w[q][c] dN[r][q]  (CSR by grid point)
 __global__ void k_resample_t(const float *__restrict__ dN, const int *__restrict__ rowptr,
-                             const int *__restrict__ col, const float *__restrict__ val, float *__restrict__ dG,
-                             int B, int ng, int nq) {
+                             const int *__restrict__ col, const float *__restrict__ val, const float *__restrict__ Y,
+                             float *__restrict__ dZ, int B, int ng, int nq) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
     if (i >= ng || r >= B) return;
     float s = 0.f;
     for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) s += val[e] * dN[(long long)r * nq + col[e]];
-    dG[(long long)r * ng + i] = s;
+    const float y = Y[(long long)r * ng + i];
+    dZ[(long long)r * ng + i] = s * (1.f - y * y);
 }
 
 // d = 2 (p - t) / (B nq); per-block partial sums of (p - t)^2 into part
@@ -325,8 +391,10 @@ struct pf_no {
     float *rw = nullptr, *rv = nullptr;
     std::vector<float *> act, dact;        // activations per layer (B x dims[l])
     float *pn = nullptr, *dn = nullptr;    // predictions and their gradient at the nodes
-    float *feat = nullptr, *targ = nullptr, *bf = nullptr, *bt = nullptr;
-    int *rows = nullptr;
+    int *order = nullptr;                  // an epoch's sample order (pf_no_train)
+    double *lpart = nullptr;               // loss partials of an epoch's batches (pf_no_train)
+    long long lpart_n = 0;
+    float *feat = nullptr, *targ = nullptr, *bt = nullptr;
     long long nsample_dev = 0;
     double *part = nullptr;
     long long adam_t = 0;
@@ -357,7 +425,6 @@ void ensure_batch(pf_no *h, int B) {
     h->pn = h->mk<float>((size_t)B * h->nq);
     h->dn = h->mk<float>((size_t)B * h->nq);
     h->bt = h->mk<float>((size_t)B * h->nq);
-    h->rows = h->mk<int>(B);
     h->maxB = B;
 }
 
@@ -400,37 +467,34 @@ void forward(pf_no *h, int B) {
     NO_CU(cudaGetLastError());
 }
 
-// loss against targets tgt (device, B x nq) and the gradient of every parameter into h->g
-double backward(pf_no *h, int B, const float *tgt) {
+// squared error against targets tgt (device, B x nq) as 256 partial sums into part (device), and the
+// gradient of every parameter into h->g
+void backward(pf_no *h, int B, const float *tgt, double *part) {
     const int L = (int)h->dims.size() - 1;
     const long long n = (long long)B * h->nq;
-    k_loss<<<256, 256, 0, h->st>>>(h->pn, tgt, h->dn, n, 1.f / (float)n, h->part);
+    k_loss<<<256, 256, 0, h->st>>>(h->pn, tgt, h->dn, n, 1.f / (float)n, part);
     NO_CU(cudaGetLastError());
-    k_resample_t<<<dim3((h->ng + 127) / 128, B), 128, 0, h->st>>>(h->dn, h->rp, h->rc, h->rv, h->dact[L], B, h->ng,
+    k_resample_t<<<dim3((h->ng + 127) / 128, B), 128, 0, h->st>>>(h->dn, h->rp, h->rc, h->rv, h->act[L], h->dact[L], B, h->ng,
                                                                   h->nq);
     NO_CU(cudaGetLastError());
     for (int l = L - 1; l >= 0; --l) {
         const int K = h->dims[l], N = h->dims[l + 1];
-        const long long nz = (long long)B * N;
-        k_tanh_back<<<(unsigned)((nz + 255) / 256), 256, 0, h->st>>>(h->act[l + 1], h->dact[l + 1], nz);
-        NO_CU(cudaGetLastError());
-        k_dense_bwd_w<<<dim3((N + 127) / 128, K), 128, 0, h->st>>>(h->act[l], h->dact[l + 1], h->g + h->woff[l],
-                                                                    h->g + h->boff[l], B, K, N,
-                                                                    l == 0 ? h->mean : nullptr,
-                                                                    l == 0 ? h->istd : nullptr);
+        k_dense_bwd_w<<<dim3((N + 127) / 128, (K + BW_K - 1) / BW_K), 128, 0, h->st>>>(
+            h->act[l], h->dact[l + 1], h->g + h->woff[l], h->g + h->boff[l], B, K, N, l == 0 ? h->mean : nullptr,
+            l == 0 ? h->istd : nullptr);
         NO_CU(cudaGetLastError());
         if (l > 0) {
-            const long long warps = (long long)B * K;
-            k_dense_bwd_x<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, h->st>>>(h->dact[l + 1], h->wb + h->woff[l],
-                                                                                   h->dact[l], B, K, N);
+            const int warps = (B + BX_T - 1) / BX_T * ((K + BX_T - 1) / BX_T);
+            k_dense_bwd_x<<<(warps + 7) / 8, 256, 0, h->st>>>(h->dact[l + 1], h->wb + h->woff[l], h->act[l], h->dact[l], B, K, N);
             NO_CU(cudaGetLastError());
         }
     }
-    std::vector<double> part(256);
-    NO_CU(cudaMemcpyAsync(part.data(), h->part, 256 * sizeof(double), cudaMemcpyDeviceToHost, h->st));
-    NO_CU(cudaStreamSynchronize(h->st));
+}
+
+// mean squared error from a batch's 256 partial sums (host)
+double mean_loss(const double *part, long long n) {
     double s = 0.0;
-    for (double v : part) s += v;
+    for (int i = 0; i < 256; ++i) s += part[i];
     return s / (double)n;
 }
 
@@ -679,7 +743,11 @@ extern "C" int pf_no_loss_grad(pf_no *h, int B, const double *feat, const double
         for (size_t i = 0; i < t.size(); ++i) t[i] = (float)target[i];
         NO_CU(cudaMemcpyAsync(h->bt, t.data(), t.size() * 4, cudaMemcpyHostToDevice, h->st));
         forward(h, B);
-        *loss = backward(h, B, h->bt);
+        backward(h, B, h->bt, h->part);
+        std::vector<double> part(256);
+        NO_CU(cudaMemcpyAsync(part.data(), h->part, 256 * sizeof(double), cudaMemcpyDeviceToHost, h->st));
+        NO_CU(cudaStreamSynchronize(h->st));
+        *loss = mean_loss(part.data(), (long long)B * h->nq);
         if (grad) {
             std::vector<float> g(h->nparam);
             NO_CU(cudaMemcpyAsync(g.data(), h->g, h->nparam * 4, cudaMemcpyDeviceToHost, h->st));
@@ -702,9 +770,15 @@ extern "C" int pf_no_train(pf_no *h, int nsample, const double *feat, const doub
         if (nsample > h->nsample_dev) {
             h->feat = h->mk<float>((size_t)nsample * F);
             h->targ = h->mk<float>((size_t)nsample * h->nq);
-            h->bf = h->mk<float>((size_t)batch * F);
+            h->order = h->mk<int>(nsample);
             h->nsample_dev = nsample;
         }
+        const int nbatch = nsample / batch;
+        if (nbatch > h->lpart_n) {
+            h->lpart = h->mk<double>((size_t)256 * nbatch);
+            h->lpart_n = nbatch;
+        }
+        std::vector<double> part((size_t)256 * std::max(1, nbatch));
         std::vector<float> f((size_t)nsample * F), t((size_t)nsample * h->nq);
         for (size_t i = 0; i < f.size(); ++i) f[i] = (float)feat[i];
         for (size_t i = 0; i < t.size(); ++i) t[i] = (float)target[i];
@@ -715,19 +789,23 @@ extern "C" int pf_no_train(pf_no *h, int nsample, const double *feat, const doub
         for (int i = 0; i < nsample; ++i) order[i] = i;
         for (int ep = 0; ep < epochs; ++ep) {
             std::shuffle(order.begin(), order.end(), rng);
-            double lsum = 0.0;
-            int nb = 0;
-            for (int s0 = 0; s0 + batch <= nsample; s0 += batch) {
-                NO_CU(cudaMemcpyAsync(h->rows, order.data() + s0, batch * sizeof(int), cudaMemcpyHostToDevice, h->st));
-                k_gather_rows<<<dim3((F + 127) / 128, batch), 128, 0, h->st>>>(h->feat, h->rows, h->act[0], batch, F);
-                k_gather_rows<<<dim3((h->nq + 127) / 128, batch), 128, 0, h->st>>>(h->targ, h->rows, h->bt, batch, h->nq);
+            // the epoch's order goes up and its losses come down once: the batches follow each other on
+            // the stream without the host
+            NO_CU(cudaMemcpyAsync(h->order, order.data(), nsample * sizeof(int), cudaMemcpyHostToDevice, h->st));
+            for (int nb = 0; nb < nbatch; ++nb) {
+                const int *rows = h->order + (size_t)nb * batch;
+                k_gather_rows<<<dim3((F + 127) / 128, batch), 128, 0, h->st>>>(h->feat, rows, h->act[0], batch, F);
+                k_gather_rows<<<dim3((h->nq + 127) / 128, batch), 128, 0, h->st>>>(h->targ, rows, h->bt, batch, h->nq);
                 NO_CU(cudaGetLastError());
                 forward(h, batch);
-                lsum += backward(h, batch, h->bt);
+                backward(h, batch, h->bt, h->lpart + (size_t)256 * nb);
                 adam(h, lr);
-                ++nb;
             }
-            if (loss_per_epoch) loss_per_epoch[ep] = nb ? lsum / nb : 0.0;
+            NO_CU(cudaMemcpyAsync(part.data(), h->lpart, (size_t)256 * nbatch * sizeof(double), cudaMemcpyDeviceToHost, h->st));
+            NO_CU(cudaStreamSynchronize(h->st));   // before `order` is shuffled again, too
+            double lsum = 0.0;
+            for (int nb = 0; nb < nbatch; ++nb) lsum += mean_loss(part.data() + (size_t)256 * nb, (long long)batch * h->nq);
+            if (loss_per_epoch) loss_per_epoch[ep] = nbatch ? lsum / nbatch : 0.0;
         }
         NO_CU(cudaStreamSynchronize(h->st));
     } catch (const NoErr &e) {
