@@ -12,7 +12,6 @@
 // The new level is written over level n-1, then the two levels swap roles.
 #include <cuda.h>
 #include <cuda_runtime.h>
-#include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cmath>
@@ -58,22 +57,7 @@ void raise_smem_limit(const void *fn, size_t bytes) {
         PF_CU(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
 }
 
-// cuTensorMapEncodeTiled from the driver, through the runtime (no link against libcuda); null when
-// the driver does not provide it
-using EncodeTiled = PFN_cuTensorMapEncodeTiled_v12000;
-EncodeTiled tc_encode() {
-    static EncodeTiled fn = [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            p = nullptr;
-        }
-        return reinterpret_cast<EncodeTiled>(p);
-    }();
-    return fn;
-}
+using pf::tc_encode;
 
 int num_sms() {
     int dev = 0, n = 0;
@@ -543,7 +527,7 @@ struct Engine {
                 add_oz(Sy[b], tr(s.Sy[b], ny), ny);
                 add_oz(SyT[b], s.Sy[b], ny);
             }
-            raise_smem_limit((const void *)pf::k_gemm_oz, OZ_SMEM);
+            raise_smem_limit((const void *)pf::k_gemm_oz, pf::OZ_SMEM);
             const long long most = (s.model == PF_MODEL_EQUILIBRIUM ? 1ll : d3 ? 3ll : 2ll) * nz;   // planes of a solve
             ozdig = mk<__half>((size_t)pf::OZ_S * most * std::max((long long)ny * oz_kpad(nx), (long long)nx * oz_kpad(ny)));
             ozE = mk<int>(most * std::max(nx, ny));
@@ -563,8 +547,7 @@ struct Engine {
     }
 
     // ---- FP64 transforms by exact digit products on the tensor cores (pf_oz.cuh) -----------------
-    static constexpr size_t OZ_SMEM = 227 * 1024;
-    static int oz_kpad(int k) { return (k + pf::OZ_KC - 1) / pf::OZ_KC * pf::OZ_KC; }
+    static int oz_kpad(int k) { return pf::oz_kpad(k); }
     // Eight launches a solve of about 5 us at least against the SIMT transforms' three or four: measured
     // per 2D step, 24 x 13 nodes 0.277 / 0.271 ms (digits / SIMT), 30 x 16 0.279 / 0.289, 48 x 25 0.310 /
     // 0.384, 240 x 121 0.571 / 1.276
@@ -617,14 +600,7 @@ struct Engine {
             if (m.ptr == ptr && m.rows == rows && m.Kpad == Kpad && m.box == box_rows) return m.map;
         OzMap m;
         m.ptr = ptr; m.rows = rows; m.Kpad = Kpad; m.box = box_rows;
-        cuuint64_t dims[3] = {(cuuint64_t)Kpad, (cuuint64_t)rows, (cuuint64_t)pf::OZ_S};
-        cuuint64_t strides[2] = {(cuuint64_t)Kpad * 2, (cuuint64_t)Kpad * 2 * rows};
-        cuuint32_t box[3] = {(cuuint32_t)pf::OZ_KC, (cuuint32_t)box_rows, (cuuint32_t)pf::OZ_S};
-        cuuint32_t estr[3] = {1, 1, 1};
-        const CUresult r = tc_encode()(&m.map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half *>(ptr), dims, strides, box,
-                                       estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled"};
+        if (!pf::oz_encode(&m.map, ptr, rows, Kpad, box_rows)) throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled"};
         ozmaps.push_back(m);
         return m.map;
     }
@@ -636,25 +612,9 @@ struct Engine {
         if (!ob) throw CudaError{cudaErrorInvalidValue, "digit-product transform without its eigenbasis"};
         if (rows >= (1ll << 31) - pf::OZ_BM) throw CudaError{cudaErrorInvalidValue, "digit-product transform with 2^31 rows"};
         if (sms == 0) sms = num_sms();
-        pf::OzArgs a{};
-        const int N = ob->n, mt = (int)((rows + pf::OZ_BM - 1) / pf::OZ_BM);
-        a.nst = ob->Kpad / pf::OZ_KC;
-        // column tiles: enough units for the chip, against the cycles of a unit: 56 MMAs a stage of
-        // 32 + N/4 cycles, about 2500 + 60 per column around them
-        double best = 0;
-        for (int nt = (N + 2 * pf::OZ_MAXH - 1) / (2 * pf::OZ_MAXH); nt <= (N + 15) / 16; ++nt) {
-            const int bn = ((N + nt - 1) / nt + 15) / 16 * 16, tiles = (N + bn - 1) / bn;
-            const double rounds = (double)(((long long)mt * tiles + sms - 1) / sms);
-            const double t = rounds * (a.nst * (56.0 * (36.0 + 0.25 * bn)) + 2500.0 + 60.0 * bn);
-            if (a.BN == 0 || t < 0.98 * best) { best = t; a.BN = bn; a.ntn = tiles; }
-        }
-        a.BNlast = ((N - (a.ntn - 1) * a.BN) + 15) / 16 * 16;
-        a.M = (int)rows; a.N = N; a.K = N;
-        a.tmem_cols = 512;
-        a.nr = std::min(pf::OZ_MAXR, 512 / a.BN) / 2 * 2;
-        const size_t stage = pf::OZ_ABYTES + (size_t)pf::OZ_S * a.BN * pf::OZ_KC * 2;
-        a.stages = (int)std::min<size_t>(4, (OZ_SMEM - pf::OZ_FIXED) / stage);
-        a.nunits = mt * a.ntn;
+        const int N = ob->n;
+        size_t smem = 0;
+        pf::OzArgs a = pf::oz_plan(rows, N, sms, &smem);
         a.E = ozE; a.F = ob->F;
         a.R = R; a.store = store; a.ldc = N; a.ldr = R;
         a.lamN = reinterpret_cast<const double *>(lamN); a.lamR = reinterpret_cast<const double *>(lamR);
@@ -668,23 +628,11 @@ struct Engine {
         const CUtensorMap ma = ozmap(ozdig, rows, ob->Kpad, pf::OZ_BM), mb = ozmap(ob->dig, N, ob->Kpad, a.BN);
         const double *A64 = reinterpret_cast<const double *>(A);
         prof->begin(PF_KC_GEMM, st);
-        const unsigned sg = (unsigned)((rows + 7) / 8);
-        auto split = [&](auto ni) {
-            pf::k_oz_split<decltype(ni)::value><<<sg, 256, 0, st>>>(A64, a.M, N, ob->Kpad, ozdig, ozE, R, active, nz);
-        };
-        switch ((ob->Kpad + 63) / 64) {
-            case 1: split(std::integral_constant<int, 1>{}); break;
-            case 2: split(std::integral_constant<int, 2>{}); break;
-            case 3: split(std::integral_constant<int, 3>{}); break;
-            case 4: split(std::integral_constant<int, 4>{}); break;
-            case 5: split(std::integral_constant<int, 5>{}); break;
-            case 6: split(std::integral_constant<int, 6>{}); break;
-            default: split(std::integral_constant<int, 8>{});
-        }
+        pf::oz_split(A64, N, 1, a.M, N, ozdig, ozE, R, active, nz, st);
         check_launch();
         prof->end(st);
         prof->begin(PF_KC_GEMM, st);
-        pf::k_gemm_oz<<<(unsigned)std::min(a.nunits, sms), pf::OZ_THREADS, a.stages * stage + pf::OZ_FIXED, st>>>(ma, mb, a);
+        pf::k_gemm_oz<<<(unsigned)std::min(a.nunits, sms), pf::OZ_THREADS, smem, st>>>(ma, mb, a);
         check_launch();
         prof->end(st);
     }

@@ -32,24 +32,25 @@ namespace pf {
 constexpr int OZ_S = 7;                       // digits per operand
 constexpr int OZ_KC = 32;                     // K per stage: 64-byte rows of FP16
 constexpr int OZ_BM = 128;                    // rows per unit = TMEM lanes
-constexpr int OZ_MAXH = 48;                   // accumulator columns per drain thread: BN <= 96
+constexpr int OZ_MAXH = 24;                   // accumulator columns per drain thread: BN <= 96
 constexpr int OZ_MAXK = 480;                  // K bound of the 64-bit sums (< 512)
 constexpr int OZ_MAXR = 16;                   // TMEM regions in the ring at most
-constexpr int OZ_EPI_WARPS = 8;
-constexpr int OZ_THREADS = 384;
-// the launch holds 384 x 168 = 64512 registers: 256 x 216 + 128 x 72 = 64512
-constexpr int OZ_REG_EPI = 216, OZ_REG_AUX = 72;
-static_assert(256 * OZ_REG_EPI + 128 * OZ_REG_AUX <= OZ_THREADS * 168, "the setmaxnreg split must fit the launch's registers");
+constexpr int OZ_EPI_WARPS = 16;              // four warpgroups: a quarter of the columns each
+constexpr int OZ_THREADS = 640;
+// the launch holds 640 x 96 = 61440 registers: 512 x 104 + 128 x 64 = 61440
+constexpr int OZ_REG_EPI = 104, OZ_REG_AUX = 64;
+static_assert(512 * OZ_REG_EPI + 128 * OZ_REG_AUX <= OZ_THREADS * 96, "the setmaxnreg split must fit the launch's registers");
+constexpr unsigned long long OZ_BIAS = 0x4B400000ull;   // bits of 1.5 2^23
 constexpr uint32_t OZ_ABYTES = OZ_S * OZ_BM * OZ_KC * 2;   // A digits of a stage
-constexpr int OZ_OUTP = 9;                    // row pitch (doubles) of a drain warp's 32 x 8 store block
+constexpr int OZ_OUTC = 4, OZ_OUTP = 5;       // columns and row pitch (doubles) of a drain warp's store block
 constexpr size_t OZ_OUTBYTES = (size_t)OZ_EPI_WARPS * 32 * OZ_OUTP * 8;
 constexpr size_t OZ_FIXED = 1024 + OZ_OUTBYTES + 512;      // alignment slack; store blocks; barriers, TMEM slot
 
 struct OzArgs {
     int M, N, K;
-    int BN;                   // column tile (multiple of 16, <= 2 OZ_MAXH)
+    int BN;                   // column tile (multiple of 32, <= 4 OZ_MAXH)
     int ntn;                  // column tiles
-    int BNlast;               // width of the last one (multiple of 16)
+    int BNlast;               // width of the last one (multiple of 32)
     int nst;                  // K stages
     int nr;                   // TMEM regions (even, nr BN <= tmem_cols)
     int stages;               // shared-memory stages
@@ -67,9 +68,48 @@ struct OzArgs {
     const double *m2x, *m2y, *face2;
     const int *active;        // ensembles: per-run flags (0 = frozen), run = p % amod; null otherwise
     int amod;
-    int *err;
+    int *err;                 // error word; null: a call without one, whose results become NaN on a time-out
     unsigned long long wait_ns;
 };
+
+constexpr size_t OZ_SMEM = 227 * 1024;
+inline int oz_kpad(int k) { return (k + OZ_KC - 1) / OZ_KC * OZ_KC; }
+
+// sizes of the product of `rows` rows with an N x N matrix: column tiles, stages, shared memory.  Column
+// tiles: enough units for the chip, against the cycles of a unit: 56 MMAs a stage of 36 + BN/4 cycles and
+// about 2500 + 60 per column around them.
+inline OzArgs oz_plan(long long rows, int N, int sms, size_t *smem) {
+    OzArgs a{};
+    const int mt = (int)((rows + OZ_BM - 1) / OZ_BM);
+    a.M = (int)rows; a.N = N; a.K = N;
+    a.nst = oz_kpad(N) / OZ_KC;
+    double best = 0;
+    for (int nt = (N + 4 * OZ_MAXH - 1) / (4 * OZ_MAXH); nt <= (N + 31) / 32; ++nt) {
+        const int bn = ((N + nt - 1) / nt + 31) / 32 * 32, tiles = (N + bn - 1) / bn;
+        const double rounds = (double)(((long long)mt * tiles + sms - 1) / sms);
+        const double t = rounds * (a.nst * (56.0 * (36.0 + 0.25 * bn)) + 2500.0 + 60.0 * bn);
+        if (a.BN == 0 || t < 0.98 * best) { best = t; a.BN = bn; a.ntn = tiles; }
+    }
+    a.BNlast = ((N - (a.ntn - 1) * a.BN) + 31) / 32 * 32;
+    a.tmem_cols = 512;
+    a.nr = (OZ_MAXR < 512 / a.BN ? OZ_MAXR : 512 / a.BN) / 2 * 2;
+    const size_t stage = OZ_ABYTES + (size_t)OZ_S * a.BN * OZ_KC * 2, fit = (OZ_SMEM - OZ_FIXED) / stage;
+    a.stages = fit < 4 ? (int)fit : 4;
+    a.nunits = mt * a.ntn;
+    *smem = a.stages * stage + OZ_FIXED;
+    return a;
+}
+
+// digit planes [OZ_S][rows][Kpad], boxes of 32 x box_rows x 7
+inline bool oz_encode(CUtensorMap *m, const __half *ptr, long long rows, int Kpad, int box_rows) {
+    cuuint64_t dims[3] = {(cuuint64_t)Kpad, (cuuint64_t)rows, (cuuint64_t)OZ_S};
+    cuuint64_t strides[2] = {(cuuint64_t)Kpad * 2, (cuuint64_t)Kpad * 2 * rows};
+    cuuint32_t box[3] = {(cuuint32_t)OZ_KC, (cuuint32_t)box_rows, (cuuint32_t)OZ_S};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return tc_encode()(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half *>(ptr), dims, strides, box, estr,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 // K-major, 64-byte swizzle, 8-row atoms of 512 bytes
 __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr) {
@@ -144,23 +184,23 @@ __device__ __forceinline__ double oz_double(long long v, int sc) {
 
 #ifndef PF_OZ_HELPERS_ONLY
 // ---- digits of A: one warp per row ----------------------------------------------------------------
-// dig[d][m][Kpad] (FP16), E[m].  Bound by its 8 bytes read and 14 written per value, most of them in L2;
+// dig[d][m][Kpad] (FP16), E[m], of the rows A[m rs + k ks].  Bound by its 8 bytes read and 14 written per value, most of them in L2;
 // a pass of its own because inside the GEMM every column tile would split the rows again (measured there:
 // 7,000 issue slots per 128 x 32 stage against 3,100 cycles of MMAs).  NI = ceil(Kpad / 64) pairs a lane.
 template <int NI>
-__global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, int M, int K, int Kpad, __half *__restrict__ dig,
-                                                  int *__restrict__ E, int R, const int *__restrict__ active, int amod) {
+__global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, long long rs, int ks, int M, int K, int Kpad,
+                                                  __half *__restrict__ dig, int *__restrict__ E, int R, const int *__restrict__ active, int amod) {
     const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (m >= M) return;
     if (active && !active[(m / R) % amod]) return;   // a frozen run's rows: their products are not used
-    const double *row = A + (long long)m * K;
+    const double *row = A + m * rs;
     double x[NI][2];
     unsigned int e = 0;
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
         const int k = 2 * (lane + 32 * i);
-        x[i][0] = k < K ? row[k] : 0.0;
-        x[i][1] = k + 1 < K ? row[k + 1] : 0.0;
+        x[i][0] = k < K ? row[(long long)k * ks] : 0.0;
+        x[i][1] = k + 1 < K ? row[(long long)(k + 1) * ks] : 0.0;
     }
 #pragma unroll
     for (int i = 0; i < NI; ++i)
@@ -190,6 +230,23 @@ __global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, 
     }
 }
 
+// launch of k_oz_split for M rows of K <= OZ_MAXK values: row pitch rs, value pitch ks (1, n for the rows and
+// columns of an n x n matrix)
+inline void oz_split(const double *A, long long rs, int ks, int M, int K, __half *dig, int *E, int R, const int *active, int amod,
+                     cudaStream_t st) {
+    const unsigned grid = (unsigned)((M + 7) / 8);
+    const int Kpad = oz_kpad(K);
+    switch ((Kpad + 63) / 64) {
+        case 1: k_oz_split<1><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
+        case 2: k_oz_split<2><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
+        case 3: k_oz_split<3><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
+        case 4: k_oz_split<4><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
+        case 5: k_oz_split<5><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
+        case 6: k_oz_split<6><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
+        default: k_oz_split<8><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod);
+    }
+}
+
 // reciprocals of the eigenvalue sums of one solve family, [mode][r][n] (0 where a sum is 0)
 static __global__ void k_oz_rcp(double *__restrict__ out, const double *__restrict__ lamN, const double *__restrict__ lamR,
                                 const double *__restrict__ shift, int modes, int nz, int R, int N) {
@@ -212,11 +269,14 @@ __device__ __forceinline__ bool oz_frozen(const OzArgs &g, int mt) {
 }
 
 // ---- the GEMM: persistent, warp-specialised; a CTA walks units of 128 rows x BN columns -------------
-//   warp 8      TMA: per 32-wide K stage the digits of A (32 x 128 x 7) and of B (32 x BN x 7), one 3D box each
-//   warps 9-10  issue the MMAs level by level (6 first; each level of a stage into a tensor-memory region
+//   warp 16     TMA: per 32-wide K stage the digits of A (32 x 128 x 7) and of B (32 x BN x 7), one 3D box each
+//   warps 17-18 issue the MMAs level by level (6 first; each level of a stage into a tensor-memory region
 //               of its own from a ring), the levels in turn between the two warps
-//   warps 0-7   drain the regions into the 64-bit integers, then convert and store (the epilogues of k_gemm)
-// setmaxnreg moves registers from warps 8-11 to the drain warps.  Every mbarrier wait is bounded as in
+//   warps 0-15  drain the regions into the 64-bit integers, then convert and store (the epilogues of
+//               k_gemm).  Sixteen, because this code overflows the schedulers' instruction caches and its
+//               fetches are shared by a scheduler's warps: with eight a level took 950 cycles of drain
+//               against 400 of MMAs
+// setmaxnreg moves registers from warps 16-19 to the drain warps.  Every mbarrier wait is bounded as in
 // pf_tc.cuh: on time-out the error word is set, copies and MMAs in flight finish (bounded), tensor memory
 // is freed and the kernel returns.
 static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_constant__ CUtensorMap tmA,
@@ -261,7 +321,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
     auto fail = [&]() {
-        if (!*abort_flag) atomicExch(g.err, TC_ERR_TIMEOUT);
+        if (!*abort_flag && g.err) atomicExch(g.err, TC_ERR_TIMEOUT);
         *abort_flag = 1;
     };
     const int ntn = g.ntn, nst = g.nst;
@@ -347,17 +407,24 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
     } else {
         // ---- drain, epilogue (warps 0-7) ------------------------------------------------------------------
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REG_EPI));
-        const int quarter = warp & 3, half = warp >> 2;
-        long long acc[OZ_MAXH];
+        const int quarter = warp & 3, half = warp >> 2;   // 32 rows; which quarter of the columns
+        // Sums of the levels plus OZ_BIAS each (below), modulo 2^64; they start at minus the biases of a
+        // unit's stages.  Code runs at about five cycles an instruction and warp here (pf_tc.cuh), so a
+        // value takes two: a packed FP32 addition that leaves the integer in the low bits, and one
+        // multiply-add into the 64-bit sum (converting and shifting took six: 900 cycles a level).
+        constexpr unsigned long long BIAS = OZ_BIAS;
+        constexpr unsigned long long BIASES = (BIAS >> 8) + BIAS + (BIAS << 8) + (BIAS << 16) + (BIAS << 24) + (BIAS << 32) + (BIAS << 40);
+        const unsigned long long acc0 = 0ull - (unsigned long long)nst * BIASES;
+        unsigned long long acc[OZ_MAXH];
 #pragma unroll
-        for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
+        for (int j = 0; j < OZ_MAXH; ++j) acc[j] = acc0;
         int r = 0;
         uint32_t rph = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < g.nunits && ok; u += gridDim.x) {
+        for (int u = blockIdx.x; u < g.nunits && (ok || !g.err); u += gridDim.x) {
             const int mt = u / ntn, nt = u - mt * ntn;
             if (oz_frozen(g, mt)) continue;
-            const int hbn = (nt == ntn - 1 ? g.BNlast : BN) >> 1;   // columns per thread (a multiple of 8)
+            const int hbn = (nt == ntn - 1 ? g.BNlast : BN) >> 2;   // columns per thread (a multiple of 8)
             const uint32_t lane0 = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * hbn);
             for (int c = 0; c < nst && ok; ++c) {
 #pragma unroll
@@ -366,18 +433,29 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t ta = lane0 + (uint32_t)(r * BN);
 #pragma unroll
-                    for (int j0 = 0; j0 < OZ_MAXH; j0 += 16) {
-                        if (j0 < hbn) {   // 16 columns (those past hbn are another half's, or none's: not used)
-                            float v[16];
-                            tmem_ld16(ta + (uint32_t)j0, v);
+                    for (int j0 = 0; j0 < OZ_MAXH; j0 += 8) {
+                        if (j0 < hbn) {
+                            float v[8];
+                            tmem_ld8(ta + (uint32_t)j0, v);
                             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                // v is an integer below 2^22: its bits after adding 1.5 2^23
-                                const int w = __float_as_int(v[j] + 12582912.f) - 0x4B400000;
-                                long long &a = acc[j0 + j];
-                                if (d == 6) a += (long long)((w + 128) >> 8);
-                                else a += (long long)w * (1ll << (8 * (5 - d)));
+                            for (int j = 0; j < 8; j += 2) {
+                                // v is an integer below 2^22: the bits of v + 1.5 2^23 are OZ_BIAS + v (level 6:
+                                // + 128 more, so that its shift by 8 rounds)
+                                const float mg = d == 6 ? 12582912.f + 128.f : 12582912.f;
+                                unsigned long long x, y, z;
+                                asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(v[j]), "f"(v[j + 1]));
+                                asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(mg));
+                                asm("add.rn.f32x2 %0, %1, %2;" : "=l"(z) : "l"(x), "l"(y));
+                                const unsigned int w0 = (unsigned int)z, w1 = (unsigned int)(z >> 32);
+                                unsigned long long &a0 = acc[j0 + j], &a1 = acc[j0 + j + 1];
+                                if (d == 6) {
+                                    a0 += (unsigned long long)(w0 >> 8);
+                                    a1 += (unsigned long long)(w1 >> 8);
+                                } else {
+                                    a0 += (unsigned long long)w0 << (8 * (5 - d));
+                                    a1 += (unsigned long long)w1 << (8 * (5 - d));
+                                }
                             }
                         }
                     }
@@ -387,64 +465,101 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                     if (++r == NR) { r = 0; rph ^= 1u; }
                 }
             }
-            if (!ok) break;
-            // ---- epilogue: eight columns per round, the rest moved down (a small loop: code is fetched at
+            if (!ok) {
+                fail();
+                if (g.err) break;
+            }
+            // ---- epilogue: four columns per round, the rest moved down (a small loop: code is fetched at
             // about five cycles an instruction here) --------------------------------------------------
             const int m0 = mt * OZ_BM + quarter * 32, m = m0 + lane, nb = nt * BN + half * hbn;
             const int em = m < g.M ? g.E[m] : 1;
             const int p = m < g.M ? m / g.R : 0, rr = m < g.M ? m - p * g.R : 0;
+            const int ncol = min(hbn, g.N - nb);
+            const int fl = lane < ncol ? g.F[nb + lane] : 1;   // the exponents of the warp's columns, one per lane
             double *ob = outb + warp * (32 * OZ_OUTP);
             double *cb = g.C + ((long long)p * g.N + nb) * g.ldr + rr;   // store 1
-            const int ncol = min(hbn, g.N - nb);
-#pragma unroll 1
-            for (int j0 = 0; j0 < ncol; j0 += 8) {
-                double v[8];
+            const bool nan = em == 0x7FF || !ok;
+            // store 0: this lane's place in a round's block, rows 8 i + lane / 4, column lane % 4
+            const int lr = lane >> 2, lc = lane & 3;
+            const double *rp[4] = {nullptr, nullptr, nullptr, nullptr};   // the reciprocals' rows
+            double rc[4] = {1.0, 1.0, 1.0, 1.0};
+            if (g.rcp) {
+                const int pl = p % g.cpl_mod, md = g.rcp_modes == 1 ? 0 : (pl == 1 ? g.cpl_mod / 2 : pl >> 1);
+                const int q = m < g.M ? md * g.R + rr : -1;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {   // units 2^56 of X Y 2^(E + F - 2154)
-                    v[j] = oz_double(acc[j], em + (j0 + j < ncol ? g.F[nb + j0 + j] : 1) - 2154 + 56);
-                    if (em == 0x7FF) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+                for (int i = 0; i < 4; ++i) {
+                    const int row = __shfl_sync(0xffffffffu, q, 8 * i + lr);
+                    if (row >= 0) {
+                        rp[i] = g.rcp + (long long)row * g.N + nb + lc;
+                        if (lc < ncol) rc[i] = *rp[i];
+                    }
+                }
+            }
+#pragma unroll 1
+            for (int j0 = 0; j0 < ncol; j0 += OZ_OUTC) {
+                double v[OZ_OUTC], rn[4] = {1.0, 1.0, 1.0, 1.0};
+                if (g.rcp) {   // the next round's reciprocals in flight during this one
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (rp[i] && j0 + OZ_OUTC + lc < ncol) rn[i] = rp[i][j0 + OZ_OUTC];
+                }
+#pragma unroll
+                for (int j = 0; j < OZ_OUTC; ++j) {   // units 2^56 of X Y 2^(E + F - 2154)
+                    v[j] = oz_double((long long)acc[j], em + __shfl_sync(0xffffffffu, fl, j0 + j) - 2154 + 56);
+                    if (nan) v[j] = __longlong_as_double(0x7FF8000000000000ll);
                 }
                 if (g.store == 1) {             // lanes hold consecutive rows: coalesced as it is
 #pragma unroll
-                    for (int j = 0; j < 8; ++j, cb += g.ldr)
+                    for (int j = 0; j < OZ_OUTC; ++j, cb += g.ldr)
                         if (m < g.M && j0 + j < ncol) *cb = v[j];
-                } else {                        // through shared memory: eight lanes per row segment of 64 bytes
+                } else {                        // through shared memory: four lanes per row segment of 32 bytes
                     __syncwarp();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) ob[lane * OZ_OUTP + j] = v[j];
+                    for (int j = 0; j < OZ_OUTC; ++j) ob[lane * OZ_OUTP + j] = v[j];
                     __syncwarp();
-                    const int n = nb + j0 + (lane & 7);
-                    const bool in = j0 + (lane & 7) < ncol;
-#pragma unroll 2
-                    for (int i = 0; i < 8; ++i) {
-                        const int row = 4 * i + (lane >> 3), mm = m0 + row;
-                        const int pp = __shfl_sync(0xffffffffu, p, row), r2 = __shfl_sync(0xffffffffu, rr, row);
-                        if (mm < g.M && in) {
-                            double x = ob[row * OZ_OUTP + (lane & 7)];
-                            if (g.rcp) {
-                                const int pl = pp % g.cpl_mod;
-                                const int md = g.rcp_modes == 1 ? 0 : (pl == 1 ? g.cpl_mod / 2 : pl >> 1);
-                                x *= g.rcp[((long long)md * g.R + r2) * g.N + n];
-                            } else if (g.lamN) {
-                                const double dd = g.lamN[n] + g.lamR[r2] + g.cpl[pp % g.cpl_mod];
-                                x = (dd != 0.0) ? x / dd : 0.0;
-                            }
-                            g.C[(long long)mm * g.ldc + n] = x;
-                            if (g.C2) {
-                                double w2 = -g.m2x[n] * g.m2y[r2] * x;
-                                if (g.face2 && r2 == 0) w2 += g.face2[(long long)pp * g.N + n];
-                                g.C2[(long long)mm * g.ldc + n] = w2;
+                    const int n = nb + j0 + lc;
+                    const bool in = j0 + lc < ncol;
+                    double *cr = g.C + (long long)(m0 + lr) * g.ldc + n;
+                    const bool plain = !g.C2 && !(g.lamN && !g.rcp);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        v[i] = ob[(8 * i + lr) * OZ_OUTP + lc];
+                        if (g.rcp) v[i] *= rc[i];
+                        rc[i] = rn[i];
+                    }
+                    if (plain) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i, cr += 8 * (long long)g.ldc)
+                            if (in && m0 + 8 * i + lr < g.M) *cr = v[i];
+                    } else {
+#pragma unroll 1
+                        for (int i = 0; i < 4; ++i, cr += 8 * (long long)g.ldc) {
+                            const int row = 8 * i + lr, mm = m0 + row;
+                            const int pp = __shfl_sync(0xffffffffu, p, row), r2 = __shfl_sync(0xffffffffu, rr, row);
+                            double x = v[0];
+#pragma unroll
+                            for (int q = 0; q < 3; ++q) v[q] = v[q + 1];
+                            if (in && mm < g.M) {
+                                if (g.lamN && !g.rcp) {
+                                    const double dd = g.lamN[n] + g.lamR[r2] + g.cpl[pp % g.cpl_mod];
+                                    x = (dd != 0.0) ? x / dd : 0.0;
+                                }
+                                *cr = x;
+                                if (g.C2) {
+                                    double w2 = -g.m2x[n] * g.m2y[r2] * x;
+                                    if (g.face2 && r2 == 0) w2 += g.face2[(long long)pp * g.N + n];
+                                    g.C2[(long long)mm * g.ldc + n] = w2;
+                                }
                             }
                         }
                     }
                 }
 #pragma unroll
-                for (int j = 0; j + 8 < OZ_MAXH; ++j) acc[j] = acc[j + 8];
+                for (int j = 0; j + OZ_OUTC < OZ_MAXH; ++j) acc[j] = acc[j + OZ_OUTC];
             }
 #pragma unroll
-            for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
+            for (int j = 0; j < OZ_MAXH; ++j) acc[j] = acc0;
         }
-        if (!ok) fail();
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

@@ -14,6 +14,8 @@
 
 #include "../../include/pf.h"
 #include "pf_kernels.cuh"
+#define PF_TC_HELPERS_ONLY
+#include "pf_oz.cuh"
 
 void pf_internal_set_error(const std::string &msg);   // pf_api.cu: message for pf_last_error(NULL)
 
@@ -22,13 +24,25 @@ namespace {
 // Two scratch planes sets of PF_STATIC_MAX_VALUES doubles each (16 MiB in total).
 static __device__ __align__(256) double g_fdm_scratch[2 * PF_STATIC_MAX_VALUES];
 
+// Digits of the right-hand sides and of the four eigenbases for the tensor-core transforms
+// (pf_oz.cuh), 43 MB in all: planes whose padded rows fit take those, others the FMA kernel.
+constexpr size_t DIG_A = (size_t)pf::OZ_S << 21, DIG_B = (size_t)pf::OZ_S * pf::OZ_MAXK * pf::OZ_MAXK;
+constexpr int DIG_ROWS = 1 << 16, DIG_MIN = 16;   // n_x, n_y >= 16: at most 2^16 rows of 2^20 values
+struct Digits {
+    __half a[DIG_A], b[4][DIG_B];
+    int E[DIG_ROWS], F[4][pf::OZ_MAXK];
+};
+static __device__ __align__(256) unsigned char g_fdm_digits[sizeof(Digits)];
+
 std::mutex g_mu;
 double *g_scratch_ptr[64] = {nullptr};   // device address of g_fdm_scratch, per device
+Digits *g_digits_ptr[64] = {nullptr};    // device address of g_fdm_digits, per device
+int g_sms[64] = {0};
 
 // Device address of the scratch array on the current device, looked up once per device.
 // Host code must not pass the symbol itself to a kernel: on the host it only names a
 // stand-in object, not device memory.
-int scratch_for_current_device(double **out) {
+int scratch_for_current_device(double **out, Digits **digits, int *sms) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) {
@@ -47,9 +61,23 @@ int scratch_for_current_device(double **out) {
             pf_internal_set_error(std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
             return PF_ECUDA;
         }
+        void *q = nullptr;
+        int n = 0;
+        e = cudaGetSymbolAddress(&q, g_fdm_digits);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute((const void *)pf::k_gemm_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pf::OZ_SMEM);
+        if (e != cudaSuccess) {
+            pf_internal_set_error(std::string("digit scratch: ") + cudaGetErrorString(e));
+            return PF_ECUDA;
+        }
+        g_digits_ptr[dev] = static_cast<Digits *>(q);
+        g_sms[dev] = n;
         g_scratch_ptr[dev] = static_cast<double *>(p);
     }
     *out = g_scratch_ptr[dev];
+    *digits = g_digits_ptr[dev];
+    *sms = g_sms[dev];
     return PF_OK;
 }
 
@@ -64,6 +92,41 @@ int launch_gemm(const double *A, const double *B, double *C, long long rows, int
         return PF_ECUDA;
     }
     return PF_OK;
+}
+
+// C = A B through the digits of A and of B's transpose (b: which of the four eigenbases)
+int launch_digits(Digits *D, int sms, const double *A, int b, double *C, long long rows, int n, int R, int store,
+                  const double *lamN, const double *lamR, const double *cpl, int cpl_mod, cudaStream_t st) {
+    size_t smem = 0;
+    pf::OzArgs a = pf::oz_plan(rows, n, sms, &smem);
+    a.E = D->E; a.F = D->F[b];
+    a.R = R; a.store = store; a.ldc = n; a.ldr = R;
+    a.lamN = lamN; a.lamR = lamR; a.cpl = cpl; a.cpl_mod = cpl_mod;
+    a.C = C;
+    a.wait_ns = 1000000000ull;
+    CUtensorMap ma, mb;
+    if (!pf::oz_encode(&ma, D->a, rows, pf::oz_kpad(n), pf::OZ_BM) || !pf::oz_encode(&mb, D->b[b], n, pf::oz_kpad(n), a.BN)) {
+        pf_internal_set_error("cuTensorMapEncodeTiled failed");
+        return PF_ECUDA;
+    }
+    pf::oz_split(A, n, 1, (int)rows, n, D->a, D->E, R, nullptr, 1, st);
+    pf::k_gemm_oz<<<(unsigned)(a.nunits < sms ? a.nunits : sms), pf::OZ_THREADS, smem, st>>>(ma, mb, a);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        pf_internal_set_error(std::string("k_gemm_oz launch: ") + cudaGetErrorString(e));
+        return PF_ECUDA;
+    }
+    return PF_OK;
+}
+
+// The tensor-core transforms take twelve launches (the eigenbases are split anew in each call: they
+// are the caller's) against four, and are the faster ones from the smallest planes measured on: 32 x 17 nodes,
+// one plane 149 -> 80 us; 128 x 65, one plane 451 -> 107 us, 64 planes 607 -> 133 us; 240 x 121, 30 planes
+// 1547 -> 170 us.
+bool digits_fit(int nx, int ny, long long total) {
+    if (nx < DIG_MIN || ny < DIG_MIN || nx > pf::OZ_MAXK || ny > pf::OZ_MAXK || pf::tc_encode() == nullptr) return false;
+    const long long P = total / ((long long)nx * ny);
+    return P * ny * pf::oz_kpad(nx) <= (1ll << 21) && P * nx * pf::oz_kpad(ny) <= (1ll << 21);
 }
 
 }  // namespace
@@ -83,11 +146,24 @@ extern "C" int pf_fdm_solve_static(int nx, int ny, int nplanes, const double *Sx
         return PF_EINVAL;
     }
     double *scratch = nullptr;
-    int rc = scratch_for_current_device(&scratch);
+    Digits *D = nullptr;
+    int sms = 0;
+    int rc = scratch_for_current_device(&scratch, &D, &sms);
     if (rc != PF_OK) return rc;
     double *W1 = scratch, *W2 = scratch + PF_STATIC_MAX_VALUES;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const long long P = nplanes;
+    if (digits_fit(nx, ny, total)) {
+        // digits of each eigenbasis by columns
+        pf::oz_split(Sx, 1, nx, nx, nx, D->b[0], D->F[0], 1, nullptr, 1, st);
+        pf::oz_split(Sy, 1, ny, ny, ny, D->b[1], D->F[1], 1, nullptr, 1, st);
+        pf::oz_split(SyT, 1, ny, ny, ny, D->b[2], D->F[2], 1, nullptr, 1, st);
+        pf::oz_split(SxT, 1, nx, nx, nx, D->b[3], D->F[3], 1, nullptr, 1, st);
+        if ((rc = launch_digits(D, sms, rhs, 0, W1, P * ny, nx, ny, 1, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
+        if ((rc = launch_digits(D, sms, W1, 1, W2, P * nx, ny, nx, 0, lam_y, lam_x, shift, nplanes, st)) != PF_OK) return rc;
+        if ((rc = launch_digits(D, sms, W2, 2, W1, P * nx, ny, nx, 1, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
+        return launch_digits(D, sms, W1, 3, out, P * ny, nx, ny, 0, nullptr, nullptr, nullptr, 1, st);
+    }
     // the same four transforms as the handle's solves: x, y (+ eigenvalue division), y^T, x^T
     if ((rc = launch_gemm(rhs, Sx, W1, P * ny, nx, ny, 1, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
     if ((rc = launch_gemm(W1, Sy, W2, P * nx, ny, nx, 0, lam_y, lam_x, shift, nplanes, st)) != PF_OK) return rc;

@@ -76,3 +76,25 @@ def test_a_non_finite_plane_leaves_the_other_alone():
     g.close()
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[0], c[0])
     assert not np.isfinite(b[1]).all() and not np.isfinite(c[1]).all()
+
+
+@pytest.mark.parametrize("mesh,planes", [((4, 2, 4), 1), ((4, 2, 8), 5), ((8, 4, 6), 1), ((12, 8, 12), 3), ((40, 2, 12), 2)])
+def test_static_solve_with_digits(mesh, planes):
+    """The allocation-free solve splits the caller's eigenbases in each call: 16 x 9 nodes (FMA kernels),
+    32 x 17 and up (digits, also where a row needs padding and K = 480), against extended precision."""
+    torch = pytest.importorskip("torch")
+    ex, ey, K = mesh
+    wl = workloads.small3d(ex=ex, ey=ey, order=K, nz=4)
+    fac = _factors(wl, native.PF_BCSET_P)
+    Sx, Lx, Sy, Ly, Mx, My = fac
+    ny, nx = len(My), len(Mx)
+    f = np.random.default_rng(ex + planes).standard_normal((planes, ny, nx))
+    t = lambda a: torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")  # noqa: E731
+    tables = [t(Sx), t(Sx.T), t(Lx), t(Sy), t(Sy.T), t(Ly)]
+    shift, rhs = t(np.full(planes, 3.5)), t((Mx[None, :] * My[:, None]) * f)
+    out = torch.empty_like(rhs)
+    native.fdm_solve_static(nx, ny, planes, *(x.data_ptr() for x in tables), shift.data_ptr(), rhs.data_ptr(),
+                            out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    ref = _extended(f, fac, 3.5).astype(np.float64)
+    assert np.linalg.norm(out.cpu().numpy() - ref) <= 1e-13 * np.linalg.norm(ref)
