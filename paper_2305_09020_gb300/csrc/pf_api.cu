@@ -179,7 +179,7 @@ struct Engine {
     bool d3;
     std::vector<void *> allocs;
     // tables
-    T *hx, *hy, *D, *Dw, *w, *Mx, *My;
+    T *hx, *hy, *sx, *sy, *D, *Dw, *w, *Mx, *My, *iMx, *iMy;
     T *Sx, *SxT, *Lx, *Sy[4], *SyT[4], *Ly[4];
     T *liftV;
     cplx<T> *tw;
@@ -345,6 +345,14 @@ struct Engine {
         d3 = !indep && nz > 1;
         hx = up(s.hx); hy = up(s.hy); D = up(s.D); Dw = up(s.Dw); w = up(s.w);
         Mx = up(s.Mx); My = up(s.My);
+        // c / v of the values as the kernels hold them, divided in the working precision
+        auto recip = [&](const std::vector<double> &v, T c) {
+            std::vector<double> r(v.size());
+            for (size_t i = 0; i < v.size(); ++i) r[i] = (double)(c / (T)v[i]);
+            return up(r);
+        };
+        sx = recip(s.hx, T(2)); sy = recip(s.hy, T(2));
+        iMx = recip(s.Mx, T(1)); iMy = recip(s.My, T(1));
         std::vector<double> tmp;
         Sx = up(s.Sx);
         tmp.assign(s.Sx.size(), 0.0);
@@ -816,7 +824,7 @@ struct Engine {
         pf::Geo<T> g;
         g.ex = ex; g.ey = ey; g.K = K; g.p = p; g.nx = nx; g.ny = ny; g.n2 = n2; g.nz = nz;
         g.epb = epb();
-        g.hx = hx; g.hy = hy; g.D = D; g.Dw = Dw; g.w = w; g.Mx = Mx; g.My = My;
+        g.hx = hx; g.hy = hy; g.sx = sx; g.sy = sy; g.iMx = iMx; g.iMy = iMy; g.D = D; g.Dw = Dw; g.w = w; g.Mx = Mx; g.My = My;
         g.active = active;
         return g;
     }
@@ -829,6 +837,8 @@ struct Engine {
         q.nu_m = (T)hs.nu_m; q.dt = (T)hs.dt; q.sigma = (T)hs.sigma; q.cos_theta = (T)hs.cos_theta;
         q.alpha = (T)alpha_of(hs, J); q.gamma0 = (T)(J == 1 ? 1.0 : 1.5); q.J = J;
         q.wetting = std::fabs(hs.cos_theta) > 1e-15 ? 1 : 0;
+        q.inv_dt = T(1) / q.dt; q.inv_2lam = T(1) / (T(2) * q.lam); q.inv_lamg = T(1) / (q.lam * q.gamma1);
+        q.inv_rho0 = T(1) / q.rho0; q.inv_nu = T(1) / q.nu_m; q.c_gradp = -T(1) / (q.nu_m * q.rho0);
         q.eps1_p = peps1; q.eps2_p = peps2; q.eps0_p = peps0;
         return q;
     }

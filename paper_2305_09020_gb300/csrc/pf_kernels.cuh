@@ -47,10 +47,12 @@ struct Geo {
     int ex, ey, K, p, nx, ny, n2, nz;
     int epb;            // elements per block of the element kernels
     const T *hx, *hy;   // element sizes
+    const T *sx, *sy;   // 2 / h of each element
     const T *D;         // D[a*p+m] = l_m'(xi_a)
     const T *Dw;        // Dw[a*p+c] = w_a D[a*p+c]
     const T *w;         // GLL weights
     const T *Mx, *My;   // assembled 1D masses
+    const T *iMx, *iMy; // their reciprocals
     const int *active;  // ensembles: per-plane (run) flag, 0 = frozen (its step is skipped); else null
 };
 
@@ -65,6 +67,8 @@ struct Phys {
     T rho1, rho2, mu1, mu2, eps1, eps2;
     T lam, inv_eta2, gamma1, S_eta2, eps0, rho0, nu_m, dt, sigma, cos_theta;
     T alpha, gamma0;
+    T inv_dt, inv_2lam, inv_lamg, inv_rho0, inv_nu, c_gradp;   // 1/dt, 1/(2 lambda), 1/(lambda gamma1), 1/rho0, 1/nu_m,
+                                                               // -1/(nu_m rho0)
     int J;
     int wetting;   // theta_s != 90 degrees
     const T *eps1_p, *eps2_p, *eps0_p;   // per-plane permittivities of an ensemble (nullable)
@@ -104,6 +108,15 @@ template <typename T> __device__ __forceinline__ T dtheta_of(const Phys<T> &q, T
 // BDF-J extrapolation xi* and the history term xi_hat (Sec. 3.1)
 template <typename T> __device__ __forceinline__ T star(int J, T a, T b) { return J == 1 ? a : T(2) * a - b; }
 template <typename T> __device__ __forceinline__ T hatv(int J, T a, T b) { return J == 1 ? a : T(2) * a - T(0.5) * b; }
+
+// x / d by the reciprocal rd = 1/d of a constant and one residual correction (Markstein): the quotient as
+// the division operator rounds it, in three operations.  The operator takes about ten, and in FP64, at two
+// operations per SM and cycle, the five to eight divisions by constants a node had were a fifth to a third
+// of the element kernels' time.
+template <typename T> __device__ __forceinline__ T divc(T x, T d, T rd) {
+    const T q = x * rd;
+    return fma(fma(-q, d, x), rd, q);
+}
 
 // ---- element helpers ----------------------------------------------------------------------
 struct ElemIdx {
@@ -293,8 +306,8 @@ __global__ void k_potential(Geo<T> G_, Phys<T> q_, const T *__restrict__ phin, c
     T c = 0;
     if (act) {
         c = eps_of(q, phis) - q.eps0;
-        sRx[e.t] = c * ddx(sV, sD, G.p, e.a, e.b, T(2) / hx);
-        sRy[e.t] = c * ddy(sV, sD, G.p, e.a, e.b, T(2) / hy);
+        sRx[e.t] = c * ddx(sV, sD, G.p, e.a, e.b, G.sx[e.ex]);
+        sRy[e.t] = c * ddy(sV, sD, G.p, e.a, e.b, G.sy[e.ey]);
     }
     __syncthreads();
     if (!act) return;
@@ -354,8 +367,8 @@ __global__ void k_efield(Geo<T> G_, const T *__restrict__ V, T *__restrict__ Ex,
             sy += G.w[bs[c]] * s;
         }
     }
-    Ex[gid] = sx / G.Mx[j];
-    Ey[gid] = sy / G.My[i];
+    Ex[gid] = divc(sx, G.Mx[j], G.iMx[j]);
+    Ey[gid] = divc(sy, G.My[i], G.iMy[i]);
 }
 
 // The same E_x, E_y (eq. 55 / 78) for FP32 runs of a compiled order: one block per element row
@@ -408,7 +421,7 @@ __global__ void __launch_bounds__(1024) k_efield_rows(Geo<float> G_, DTab<KC> t,
 #pragma unroll
             for (int m = 0; m < P; ++m) s += t.d[b * P + m] * c[m];
             sy += t.w[b] * s;
-            Eyp[(long long)(r0 + b) * nx] = sy / G.My[r0 + b];
+            Eyp[(long long)(r0 + b) * nx] = divc(sy, G.My[r0 + b], G.iMy[r0 + b]);
         }
     }
     __syncthreads();
@@ -438,7 +451,7 @@ __global__ void __launch_bounds__(1024) k_efield_rows(Geo<float> G_, DTab<KC> t,
                 for (int m = 0; m < P; ++m) sl += t.d[K * P + m] * vl[m];
                 sx += t.w[K] * sl;
             }
-            sE[r * nx + e * K + a] = sx / G.Mx[e * K + a];
+            sE[r * nx + e * K + a] = divc(sx, G.Mx[e * K + a], G.iMx[e * K + a]);
         }
     }
     __syncthreads();
@@ -473,13 +486,13 @@ __global__ void k_chem(Geo<T> G_, Phys<T> q_, const T *__restrict__ phin, const 
         sP[e.t] = phis;
         const T ex = Ex[e.g], ey = Ey[e.g], ez = Ez ? Ez[e.g] : T(0);
         const T E2 = ex * ex + ey * ey + ez * ez;
-        const T Q2 = h_of(q, phis) - q.S_eta2 * phis - deps_of(q, phis) / (T(2) * q.lam) * E2;
+        const T Q2 = h_of(q, phis) - q.S_eta2 * phis - divc(deps_of(q, phis), T(2) * q.lam, q.inv_2lam) * E2;
         sQ[e.t] = Q2;
         Q2n[e.g] = Q2;   // identical value from every element sharing the node
     }
     __syncthreads();
     if (act) {
-        const T sx = T(2) / hx, sy = T(2) / hy;
+        const T sx = G.sx[e.ex], sy = G.sy[e.ey];
         const T *fs[2] = {sP, sQ};   // phi* and Q2, each coefficient loaded once for both
         T dx[2], dy[2];
         ddx_n(fs, sD, G.p, e.a, e.b, sx, dx);
@@ -489,7 +502,7 @@ __global__ void k_chem(Geo<T> G_, Phys<T> q_, const T *__restrict__ phin, const 
         T adv = star(q.J, uxn[e.g], uxo[e.g]) * gpx + star(q.J, uyn[e.g], uyo[e.g]) * gpy;
         if (uzn) adv += star(q.J, uzn[e.g], uzo[e.g]) * star(q.J, dzphin[e.g], dzphio[e.g]);
         const T phh = hatv(q.J, phin[e.g], phio[e.g]);
-        Q1 = (-adv + phh / q.dt) / (q.lam * q.gamma1);
+        Q1 = divc(-adv + divc(phh, q.dt, q.inv_dt), q.lam * q.gamma1, q.inv_lamg);
         sQx[e.t] = dx[1];
         sQy[e.t] = dy[1];
     }
@@ -557,7 +570,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_momentum(Geo<T>
     __syncthreads();
     T mr = 0, om[3] = {0, 0, 0}, Gv[3] = {0, 0, 0};
     if (act) {
-        const T sx = T(2) / hx, sy = T(2) / hy;
+        const T sx = G.sx[e.ex], sy = G.sy[e.ey];
         const T phi = sphi[e.t];
         // x and y derivatives of phi, W, u*_x, u*_y, u*_z (0 in 2D), P*, each coefficient loaded once
         const T *fs[6] = {sphi, sW, sux, suy, suz, sPs};
@@ -599,7 +612,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_momentum(Geo<T>
                 jgu += cJ * gW[d] * gu[c][d];
                 conv += us[d] * gu[c][d];
             }
-            Tv[c] = (kf * gphi[c] + visc - jgu) * irho + uh[c] / q.dt - conv + (T(1) / q.rho0 - irho) * gP[c];
+            Tv[c] = (kf * gphi[c] + visc - jgu) * irho + divc(uh[c], q.dt, q.inv_dt) - conv + (q.inv_rho0 - irho) * gP[c];
         }
         om[0] = gu[2][1] - gu[1][2];
         om[1] = gu[0][2] - gu[2][0];
@@ -624,7 +637,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_momentum(Geo<T>
     if (!act) return;
     const T hx2 = T(0.5) * hx, hy2 = T(0.5) * hy;
     const T Me = hx2 * hy2 * sw[e.a] * sw[e.b];
-    const T inu = T(1) / q.nu_m;
+    const T inu = q.inv_nu;
     const int p = G.p;
     // pressure: rho0 int G_2D . grad q - rho0 int_wall J_x dq/dx  ;  iB part: -rho0 int G_z q + rho0 int_wall J_z q
     // weak x derivatives of G_x, K_z, K_y and weak y derivatives of G_y, K_z, K_x, each coefficient
@@ -677,9 +690,9 @@ __global__ void k_ugradp(Geo<T> G_, Phys<T> q, const T *__restrict__ P, T *__res
     if (!act) return;
     const T hx = G.hx[e.ex], hy = G.hy[e.ey];
     const T Me = T(0.25) * hx * hy * sw[e.a] * sw[e.b];
-    const T c = -T(1) / (q.nu_m * q.rho0);
-    AUx[e.l] += c * Me * ddx(sPv, sD, G.p, e.a, e.b, T(2) / hx);
-    AUy[e.l] += c * Me * ddy(sPv, sD, G.p, e.a, e.b, T(2) / hy);
+    const T c = q.c_gradp;
+    AUx[e.l] += c * Me * ddx(sPv, sD, G.p, e.a, e.b, G.sx[e.ex]);
+    AUy[e.l] += c * Me * ddy(sPv, sD, G.p, e.a, e.b, G.sy[e.ey]);
     if (BUz) BUz[e.l] = c * Me * sPv[e.t];
 }
 
@@ -895,53 +908,108 @@ __device__ __forceinline__ void fft256_warp(cplx<T> *buf, int ld, int npen, cons
     __syncthreads();
 }
 
+// R-point DFT of v in place, natural order (R = 2, 3, 4, 5, 7): the real and imaginary parts of a pair of
+// outputs s, R - s are sums of cosines of v_r + v_{R-r} and of sines of v_r - v_{R-r}.  ct, st: cos and sin
+// of 2 pi m / R, m = 1 .. R/2; sg = -1 forward, +1 inverse.
+template <int R, typename T>
+__device__ __forceinline__ void dft_small(cplx<T> *v, const T *ct, const T *st, T sg) {
+    if constexpr (R == 2) {
+        const cplx<T> a = v[0], b = v[1];
+        v[0] = {a.x + b.x, a.y + b.y};
+        v[1] = {a.x - b.x, a.y - b.y};
+    } else if constexpr (R == 4) {
+        const cplx<T> a = {v[0].x + v[2].x, v[0].y + v[2].y}, b = {v[0].x - v[2].x, v[0].y - v[2].y};
+        const cplx<T> c = {v[1].x + v[3].x, v[1].y + v[3].y}, d = {v[1].x - v[3].x, v[1].y - v[3].y};
+        v[0] = {a.x + c.x, a.y + c.y};
+        v[2] = {a.x - c.x, a.y - c.y};
+        v[1] = {b.x - sg * d.y, b.y + sg * d.x};
+        v[3] = {b.x + sg * d.y, b.y - sg * d.x};
+    } else {
+        constexpr int H = R / 2;
+        cplx<T> p[H], m[H], o[R];
+        o[0] = v[0];
+#pragma unroll
+        for (int r = 0; r < H; ++r) {
+            p[r] = {v[r + 1].x + v[R - 1 - r].x, v[r + 1].y + v[R - 1 - r].y};
+            m[r] = {v[r + 1].x - v[R - 1 - r].x, v[r + 1].y - v[R - 1 - r].y};
+            o[0].x += p[r].x;
+            o[0].y += p[r].y;
+        }
+#pragma unroll
+        for (int s = 1; s <= H; ++s) {
+            cplx<T> a = v[0], b = {T(0), T(0)};
+#pragma unroll
+            for (int r = 1; r <= H; ++r) {
+                const int q = (r * s) % R, h = q <= H ? q : R - q;   // cos even, sin odd in q
+                a.x += ct[h - 1] * p[r - 1].x;
+                a.y += ct[h - 1] * p[r - 1].y;
+                const T sn = q <= H ? st[h - 1] : -st[h - 1];
+                b.x += sn * m[r - 1].x;
+                b.y += sn * m[r - 1].y;
+            }
+            o[s] = {a.x - sg * b.y, a.y + sg * b.x};
+            o[R - s] = {a.x + sg * b.y, a.y - sg * b.x};
+        }
+#pragma unroll
+        for (int s = 0; s < R; ++s) v[s] = o[s];
+    }
+}
+
+// one Stockham stage of radix R: inputs x[j + r n/R] of each pencil, twiddled by w^(r (j mod Ns) n/(Ns R)),
+// through an R-point DFT into the outputs (j / Ns) Ns R + (j mod Ns) + s Ns
+template <int R, typename T>
+__device__ __forceinline__ void fft_mixed_stage(const cplx<T> *in, cplx<T> *out, int ld, int npen, int n, int Ns,
+                                                const cplx<T> *tw, bool inverse) {
+    const int h = n / 2, nb = n / R, tstep = n / (Ns * R);
+    const T sg = inverse ? T(1) : T(-1);
+    constexpr double C[8][3] = {{}, {}, {-1.0}, {-0.5}, {0.0, -1.0},
+                                {0.30901699437494742410, -0.80901699437494742410}, {},
+                                {0.62348980185873353053, -0.22252093395631440429, -0.90096886790241912624}};
+    constexpr double S[8][3] = {{}, {}, {0.0}, {0.86602540378443864676}, {1.0, 0.0},
+                                {0.95105651629515357212, 0.58778525229247312917}, {},
+                                {0.78183148246802980871, 0.97492791218182360702, 0.43388373911755812048}};
+    const T ct[3] = {(T)C[R][0], (T)C[R][1], (T)C[R][2]}, st[3] = {(T)S[R][0], (T)S[R][1], (T)S[R][2]};
+    for (int t = threadIdx.x; t < npen * nb; t += blockDim.x) {
+        const int pen = t / nb, j = t - pen * nb, q = j / Ns, k = j - q * Ns;
+        const cplx<T> *x = in + pen * ld;
+        cplx<T> v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = x[j + r * nb];
+        if (k) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) {
+                const int m = r * k * tstep;
+                cplx<T> w = tw[m < h ? m : m - h];
+                if (m >= h) w = {-w.x, -w.y};
+                if (inverse) w.y = -w.y;
+                v[r] = cmul(v[r], w);
+            }
+        }
+        dft_small<R>(v, ct, st, sg);
+        cplx<T> *y = out + pen * ld + q * Ns * R + k;
+#pragma unroll
+        for (int s = 0; s < R; ++s) y[s * Ns] = v[s];
+    }
+    __syncthreads();
+}
+
 // Stockham autosort FFT of npen pencils of any even length n = 2^a 3^b 5^c 7^d (natural order in
-// and out; the result ends in buf, tmp is scratch of the same shape).  Each stage of radix R
-// (4, 2, 3, 5 or 7, taken in that order while it divides what is left) combines R inputs
-// x[j + r n/R] of the pencil, twiddled by w^(r (j mod Ns) n/(Ns R)), through an R-point DFT into
-// the outputs (j / Ns) Ns R + (j mod Ns) + s Ns, Ns = product of the earlier radices.  Twiddles
-// w^m = exp(-+2 pi i m / n) come from the half table tw (w^(m + n/2) = -w^m).
+// and out; the result ends in buf, tmp is scratch of the same shape), stages of radix 4, 2, 3, 5 or 7
+// taken in that order while they divide what is left.  Twiddles w^m = exp(-+2 pi i m / n) come from the
+// half table tw (w^(m + n/2) = -w^m).  Each radix has its own DFT (26 operations a value for n = 120; one
+// loop over the R x R products of twiddles took 65, and FP64 runs at two operations per SM and cycle).
 template <typename T>
 __device__ void fft_pencils_mixed(cplx<T> *buf, cplx<T> *tmp, int ld, int npen, int n, const cplx<T> *tw,
                                   bool inverse) {
-    const int h = n / 2;
-    auto W = [&](int m) {
-        cplx<T> w = m < h ? tw[m] : cplx<T>{-tw[m - h].x, -tw[m - h].y};
-        if (inverse) w.y = -w.y;
-        return w;
-    };
     cplx<T> *in = buf, *out = tmp;
     int Ns = 1, rem = n;
     while (rem > 1) {
-        const int R = (rem % 4 == 0) ? 4 : (rem % 2 == 0) ? 2 : (rem % 3 == 0) ? 3 : (rem % 5 == 0) ? 5 : 7;
-        const int nb = n / R, tstep = n / (Ns * R), sstep = n / R;
-        for (int t = threadIdx.x; t < npen * nb; t += blockDim.x) {
-            const int pen = t / nb, j = t - pen * nb, k = j % Ns;
-            const cplx<T> *x = in + pen * ld;
-            cplx<T> *y = out + pen * ld;
-            cplx<T> v[7];
-#pragma unroll
-            for (int r = 0; r < 7; ++r) {
-                if (r >= R) break;
-                v[r] = x[j + r * nb];
-                if (r) v[r] = cmul(v[r], W(r * k * tstep));
-            }
-            const int o = (j / Ns) * Ns * R + k;
-#pragma unroll
-            for (int s = 0; s < 7; ++s) {
-                if (s >= R) break;
-                cplx<T> acc = v[0];
-#pragma unroll
-                for (int r = 1; r < 7; ++r) {
-                    if (r >= R) break;
-                    const cplx<T> p = cmul(v[r], W(((r * s) % R) * sstep));
-                    acc.x += p.x;
-                    acc.y += p.y;
-                }
-                y[o + s * Ns] = acc;
-            }
-        }
-        __syncthreads();
+        int R;
+        if (rem % 4 == 0) { R = 4; fft_mixed_stage<4>(in, out, ld, npen, n, Ns, tw, inverse); }
+        else if (rem % 2 == 0) { R = 2; fft_mixed_stage<2>(in, out, ld, npen, n, Ns, tw, inverse); }
+        else if (rem % 3 == 0) { R = 3; fft_mixed_stage<3>(in, out, ld, npen, n, Ns, tw, inverse); }
+        else if (rem % 5 == 0) { R = 5; fft_mixed_stage<5>(in, out, ld, npen, n, Ns, tw, inverse); }
+        else { R = 7; fft_mixed_stage<7>(in, out, ld, npen, n, Ns, tw, inverse); }
         cplx<T> *sw = in;
         in = out;
         out = sw;
@@ -1087,18 +1155,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 2) k_fwd(Geo<T> G, F
         if (pow2) fft_pencils(buf, ld, tp, nz, stw, false);
         else fft_pencils_mixed(buf, tmp, ld, tp, nz, stw, false);
     }
-    const T inv_n = T(1) / T(nz);
-    for (int idx = threadIdx.x; idx < tp * nz; idx += blockDim.x) {
-        const int p = idx >> lgtp, ql = idx & (tp - 1), qg = q0 + ql;
+    // a thread per mode writes both of its packed planes (a thread per plane formed the spectra twice)
+    const T hn = T(0.5) / T(nz);
+    const int nk = nz > 1 ? nz / 2 + 1 : 1;
+    for (int idx = threadIdx.x; idx < tp * nk; idx += blockDim.x) {
+        const int k = idx >> lgtp, ql = idx & (tp - 1), qg = q0 + ql;
         if (qg >= G.n2) continue;
-        int k, im;
-        plane_mode(p, nz, k, im);
         const cplx<T> zk = buf[ql * ld + k];
-        const cplx<T> zn = buf[ql * ld + ((nz - k) % nz)];
+        const cplx<T> zn = buf[ql * ld + (k == 0 ? 0 : nz - k)];
         // spectra of the two real inputs
-        const cplx<T> X0 = {T(0.5) * (zk.x + zn.x) * inv_n, T(0.5) * (zk.y - zn.y) * inv_n};
-        const cplx<T> X1 = {T(0.5) * (zk.y + zn.y) * inv_n, -T(0.5) * (zk.x - zn.x) * inv_n};
+        const cplx<T> X0 = {hn * (zk.x + zn.x), hn * (zk.y - zn.y)};
+        const cplx<T> X1 = {hn * (zk.y + zn.y), -hn * (zk.x - zn.x)};
         cplx<T> R = X0;
+        const int i = qg / G.nx, j = qg - i * G.nx;
         if (a.X1) {
             const T beta = a.two_pi_over_lz * T(k);
             if (a.mult == 0) {
@@ -1106,23 +1175,27 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 2) k_fwd(Geo<T> G, F
                 R.x -= b * X1.y;
                 R.y += b * X1.x;
             } else {
-                const int i = qg / G.nx, j = qg % G.nx;
                 const T m = beta * beta * G.Mx[j] * G.My[i];
                 R.x += m * X1.x;
                 R.y += m * X1.y;
             }
         }
-        T v = a.scale * (im ? R.y : R.x);
-        if (p == 0 && a.lift) {
-            const int i = qg / G.nx, j = qg % G.nx;
-            v -= a.lift[i] * G.Mx[j];
-        }
+        const bool two = k != 0 && k != nz / 2;                  // modes 0 and nz/2 are real
+        const int p = k == 0 ? 0 : (two ? 2 * k : 1);
+        T v = a.scale * R.x, w = a.scale * R.y;
+        if (p == 0 && a.lift) v -= a.lift[i] * G.Mx[j];
         if (a.lift2y) {
-            const int i = qg / G.nx, j = qg % G.nx;
-            v -= a.lift2y[i] * G.Mx[j] * a.lift2x[(long long)p * G.nx + j];
+            const T ly = a.lift2y[i] * G.Mx[j];
+            v -= ly * a.lift2x[(long long)p * G.nx + j];
+            if (two) w -= ly * a.lift2x[(long long)(p + 1) * G.nx + j];
         }
-        a.out[(long long)p * G.n2 + qg] = v;
-        if (a.out1) a.out1[(long long)p * G.n2 + qg] = im ? X1.y : X1.x;
+        const long long o = (long long)p * G.n2 + qg;
+        a.out[o] = v;
+        if (two) a.out[o + G.n2] = w;
+        if (a.out1) {
+            a.out1[o] = X1.x;
+            if (two) a.out1[o + G.n2] = X1.y;
+        }
     }
 }
 
