@@ -117,6 +117,23 @@ T *dupload(const std::vector<double> &v, cudaStream_t st) {
     return d;
 }
 
+// Launch with the programmatic-dependent-launch attribute (for kernels that begin with pf::pdl_enter) or
+// without it
+template <typename... P, typename... Q>
+void launch(bool pdl, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Q &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    PF_CU(cudaLaunchKernelEx(&cfg, k, std::forward<Q>(args)...));
+}
+
 // Per-class launch counters and optional CUDA-event timers of the kernels a handle launches.
 struct Prof {
     bool on = false;
@@ -636,11 +653,11 @@ struct Engine {
         const CUtensorMap ma = ozmap(ozdig, rows, ob->Kpad, pf::OZ_BM), mb = ozmap(ob->dig, N, ob->Kpad, a.BN);
         const double *A64 = reinterpret_cast<const double *>(A);
         prof->begin(PF_KC_GEMM, st);
-        pf::oz_split(A64, N, 1, a.M, N, ozdig, ozE, R, active, nz, st);
+        pf::oz_split(A64, N, 1, a.M, N, ozdig, ozE, R, active, nz, st, pdl());
         check_launch();
         prof->end(st);
         prof->begin(PF_KC_GEMM, st);
-        pf::k_gemm_oz<<<(unsigned)std::min(a.nunits, sms), pf::OZ_THREADS, smem, st>>>(ma, mb, a);
+        launch(pdl(), pf::k_gemm_oz, dim3((unsigned)std::min(a.nunits, sms)), dim3(pf::OZ_THREADS), smem, st, ma, mb, a);
         check_launch();
         prof->end(st);
     }
@@ -771,7 +788,7 @@ struct Engine {
         if (sms == 0) sms = num_sms();
         const unsigned grid = (unsigned)std::min(a.ntiles, sms);
         prof->begin(PF_KC_GEMM, st);
-        pf::k_gemm_tc<<<grid, pf::TC_THREADS, tb->smem, st>>>(ma, tb->mh, tb->ml, mc, a);
+        launch(pdl(), pf::k_gemm_tc, dim3(grid), dim3(pf::TC_THREADS), tb->smem, st, ma, tb->mh, tb->ml, mc, a);
         check_launch();
         prof->end(st);
     }
@@ -844,8 +861,16 @@ struct Engine {
     }
 
     // ---- launch helpers -----------------------------------------------------------------
-    // element kernels: as many whole elements as fit in 256 threads per block
-    int epb() const { return std::max(1, 256 / (p * p)); }
+    // the kernels of a single run follow each other with programmatic dependent launches; an ensemble's
+    // groups fork from and join into other streams and keep full dependencies
+    bool pdl() const { return !indep; }
+    // element kernels: as many whole elements as fit in 256 threads per block, fewer where that leaves SMs
+    // without a block (2D, 32 elements of order 6 in FP64: the momentum kernel's five elements on one SM
+    // took 26 us at two FP64 operations per cycle, one element on each of 32 SMs takes 19)
+    int epb() const {
+        const long long spread = (long long)ex * ey * nz / 152;
+        return (int)std::max<long long>(1, std::min<long long>(256 / (p * p), spread));
+    }
     int elem_threads() const { return ((epb() * p * p + 31) / 32) * 32; }
     size_t elem_smem(int nfields) const {
         return (size_t)(2 * p * p + 32 + (size_t)epb() * nfields * p * p) * sizeof(T);
@@ -861,12 +886,12 @@ struct Engine {
     }
     void launch_inv(dim3 grid, size_t smem, const pf::InvArgs<T> &a) {
         switch (lgz()) {
-            case 4: pf::k_inv<T, 4><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 5: pf::k_inv<T, 5><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 6: pf::k_inv<T, 6><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 7: pf::k_inv<T, 7><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 8: pf::k_inv<T, 8><<<grid, 256, smem, st>>>(geo(), a); break;
-            default: pf::k_inv<T, 0><<<grid, 256, smem, st>>>(geo(), a);
+            case 4: launch(pdl(), pf::k_inv<T, 4>, grid, dim3(256), smem, st, geo(), a); break;
+            case 5: launch(pdl(), pf::k_inv<T, 5>, grid, dim3(256), smem, st, geo(), a); break;
+            case 6: launch(pdl(), pf::k_inv<T, 6>, grid, dim3(256), smem, st, geo(), a); break;
+            case 7: launch(pdl(), pf::k_inv<T, 7>, grid, dim3(256), smem, st, geo(), a); break;
+            case 8: launch(pdl(), pf::k_inv<T, 8>, grid, dim3(256), smem, st, geo(), a); break;
+            default: launch(pdl(), pf::k_inv<T, 0>, grid, dim3(256), smem, st, geo(), a);
         }
     }
     // transform buffers of a non-power-of-two nz need a second (scratch) copy for the mixed radices
@@ -880,7 +905,8 @@ struct Engine {
     static constexpr size_t FFT_SMEM_LIMIT = 96 * 1024;   // raised once per kernel at set-up
     int fwd_tp() const {
         int tp = (int)((nz_pow2() ? FFT_SMEM_BUDGET : FFT_SMEM_BUDGET / 2) / (sizeof(cplx<T>) * fld()));
-        const int by_grid = tp_override > 0 ? tp_override : n2 / (4 * 152);
+        // one plane: a block's 256 threads have a node each at most, so one block per SM rather than four
+        const int by_grid = tp_override > 0 ? tp_override : n2 / ((nz == 1 ? 1 : 4) * 152);
         if (tp > by_grid) tp = by_grid;
         if (tp > 64) tp = 64;
         if (tp < 4) tp = 4;
@@ -1088,18 +1114,18 @@ struct Engine {
         a.cs_x0 = x0l ? NL : N; a.cs_x1 = x1l ? NL : N; a.cs_out = N;
         a.X0 = X0; a.x0_local = x0l; a.X1 = X1; a.x1_local = x1l; a.mult = mult; a.scale = (T)scale;
         a.lift = lift; a.out = out; a.out1 = out1; a.two_pi_over_lz = (T)(2.0 * M_PI / hs.lz);
-        a.tw = tw; a.tp = fwd_tp();
+        a.tw = tw; a.tp = fwd_tp(); a.hn = T(0.5) / T(nz);
         const size_t smem = (size_t)((nz > 1 ? nz / 2 : 1) + a.tp * fld()) * sizeof(cplx<T>) + a.tp * 4 * sizeof(int) +
                             fft_scratch(a.tp);
         prof->begin(PF_KC_FWD, st);
         const dim3 grid((n2 + a.tp - 1) / a.tp, ncomp);
         switch (lgz()) {
-            case 4: pf::k_fwd<T, 4><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 5: pf::k_fwd<T, 5><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 6: pf::k_fwd<T, 6><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 7: pf::k_fwd<T, 7><<<grid, 256, smem, st>>>(geo(), a); break;
-            case 8: pf::k_fwd<T, 8><<<grid, 256, smem, st>>>(geo(), a); break;
-            default: pf::k_fwd<T, 0><<<grid, 256, smem, st>>>(geo(), a);
+            case 4: launch(pdl(), pf::k_fwd<T, 4>, grid, dim3(256), smem, st, geo(), a); break;
+            case 5: launch(pdl(), pf::k_fwd<T, 5>, grid, dim3(256), smem, st, geo(), a); break;
+            case 6: launch(pdl(), pf::k_fwd<T, 6>, grid, dim3(256), smem, st, geo(), a); break;
+            case 7: launch(pdl(), pf::k_fwd<T, 7>, grid, dim3(256), smem, st, geo(), a); break;
+            case 8: launch(pdl(), pf::k_fwd<T, 8>, grid, dim3(256), smem, st, geo(), a); break;
+            default: launch(pdl(), pf::k_fwd<T, 0>, grid, dim3(256), smem, st, geo(), a);
         }
         check_launch();
         prof->end(st);
@@ -1162,7 +1188,7 @@ struct Engine {
         auto q = phys(J);
         prof->begin(PF_KC_POTENTIAL, st);
         by_order([&](auto kc) {
-            pf::k_potential<T, decltype(kc)::value><<<elem_grid(), elem_threads(), elem_smem(3), st>>>(
+            launch(pdl(), pf::k_potential<T, decltype(kc)::value>, elem_grid(), dim3(elem_threads()), elem_smem(3), st,
                 G, q, phin, phio, Vn, Vo, Ezn, Ezo, LA, d3 ? LB : nullptr);
         });
         check_launch();
@@ -1212,11 +1238,11 @@ struct Engine {
                     for (int i = 0; i < (KC + 1) * (KC + 1); ++i) t.d[i] = (float)hs.D[i];
                     for (int i = 0; i <= KC; ++i) t.w[i] = (float)hs.w[i];
                     const unsigned thr = (unsigned)std::min(1024, (nx + 31) / 32 * 32);
-                    pf::k_efield_rows<KC><<<dim3(ey, nz), thr, rows_smem, st>>>(geo(), t, Vf, Ex, Ey);
+                    launch(pdl(), pf::k_efield_rows<KC>, dim3(ey, nz), dim3(thr), rows_smem, st, geo(), t, Vf, Ex, Ey);
                     return;
                 }
             }
-            pf::k_efield<T, KC><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(geo(), Vf, Ex, Ey);
+            launch(pdl(), pf::k_efield<T, KC>, dim3((unsigned)((tot + 255) / 256)), dim3(256), 0, st, geo(), Vf, Ex, Ey);
         });
         check_launch();
         prof->end(st);
@@ -1234,7 +1260,7 @@ struct Engine {
         // psi^{n+1}
         prof->begin(PF_KC_CHEM, st);
         by_order([&](auto kc) {
-            pf::k_chem<T, decltype(kc)::value><<<elem_grid(), elem_threads(), elem_smem(4), st>>>(
+            launch(pdl(), pf::k_chem<T, decltype(kc)::value>, elem_grid(), dim3(elem_threads()), elem_smem(4), st,
                 G, q, phi[n], phi[o], dzphi[n], dzphi[o], u[0][n], u[0][o], u[1][n], u[1][o], u[2][n], u[2][o], Ex,
                 Ey, Ez[o], LA, Q2, q.wetting ? faceU : nullptr);
         });
@@ -1284,7 +1310,7 @@ struct Engine {
         for (int c = 0; c < 3; ++c) { mo.AU[c] = LAU[c]; mo.BU[c] = LBU[c]; }
         prof->begin(PF_KC_MOMENTUM, st);
         by_order([&](auto kc) {
-            pf::k_momentum<T, decltype(kc)::value><<<elem_grid(), elem_threads(), elem_smem(12), st>>>(G, q, mi, mo);
+            launch(pdl(), pf::k_momentum<T, decltype(kc)::value>, elem_grid(), dim3(elem_threads()), elem_smem(12), st, G, q, mi, mo);
         });
         check_launch();
         prof->end(st);
@@ -1296,7 +1322,7 @@ struct Engine {
         // u^{n+1}
         prof->begin(PF_KC_UGRADP, st);
         by_order([&](auto kc) {
-            pf::k_ugradp<T, decltype(kc)::value><<<elem_grid(), elem_threads(), elem_smem(1), st>>>(
+            launch(pdl(), pf::k_ugradp<T, decltype(kc)::value>, elem_grid(), dim3(elem_threads()), elem_smem(1), st,
                 G, q, P[o], LAU[0], LAU[1], d3 ? LBU[2] : nullptr);
         });
         check_launch();

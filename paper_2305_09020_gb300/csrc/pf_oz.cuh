@@ -191,6 +191,7 @@ template <int NI>
 __global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, long long rs, int ks, int M, int K, int Kpad,
                                                   __half *__restrict__ dig, int *__restrict__ E, int R, const int *__restrict__ active, int amod) {
     const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    tc_pdl_enter();
     if (m >= M) return;
     if (active && !active[(m / R) % amod]) return;   // a frozen run's rows: their products are not used
     const double *row = A + m * rs;
@@ -231,19 +232,30 @@ __global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, 
 }
 
 // launch of k_oz_split for M rows of K <= OZ_MAXK values: row pitch rs, value pitch ks (1, n for the rows and
-// columns of an n x n matrix)
+// columns of an n x n matrix); pdl: as a programmatic dependent launch
 inline void oz_split(const double *A, long long rs, int ks, int M, int K, __half *dig, int *E, int R, const int *active, int amod,
-                     cudaStream_t st) {
-    const unsigned grid = (unsigned)((M + 7) / 8);
+                     cudaStream_t st, bool pdl = false) {
     const int Kpad = oz_kpad(K);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((M + 7) / 8));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    auto go = [&](void (*k)(const double *, long long, int, int, int, int, __half *, int *, int, const int *, int)) {
+        cudaLaunchKernelEx(&cfg, k, A, rs, ks, M, K, Kpad, dig, E, R, active, amod);   // errors: the caller's cudaGetLastError
+    };
     switch ((Kpad + 63) / 64) {
-        case 1: k_oz_split<1><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
-        case 2: k_oz_split<2><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
-        case 3: k_oz_split<3><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
-        case 4: k_oz_split<4><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
-        case 5: k_oz_split<5><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
-        case 6: k_oz_split<6><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod); break;
-        default: k_oz_split<8><<<grid, 256, 0, st>>>(A, rs, ks, M, K, Kpad, dig, E, R, active, amod);
+        case 1: go(k_oz_split<1>); break;
+        case 2: go(k_oz_split<2>); break;
+        case 3: go(k_oz_split<3>); break;
+        case 4: go(k_oz_split<4>); break;
+        case 5: go(k_oz_split<5>); break;
+        case 6: go(k_oz_split<6>); break;
+        default: go(k_oz_split<8>);
     }
 }
 
@@ -320,6 +332,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
+    tc_pdl_enter();   // everything above is this kernel's own
     auto fail = [&]() {
         if (!*abort_flag && g.err) atomicExch(g.err, TC_ERR_TIMEOUT);
         *abort_flag = 1;

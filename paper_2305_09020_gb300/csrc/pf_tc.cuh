@@ -280,6 +280,13 @@ __device__ __forceinline__ void div_cols(float *acc, const float *lam, float lr)
     }
 }
 
+// Programmatic dependent launch (pf_kernels.cuh: pdl_enter): the GEMMs let their successor start at once,
+// as their few CTAs leave room for it
+__device__ __forceinline__ void tc_pdl_enter() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 #ifndef PF_TC_HELPERS_ONLY   // translation units that only need the helpers above
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBh,
@@ -323,6 +330,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    tc_pdl_enter();   // everything above is this kernel's own
     if (g.stall) {   // test hook: nothing arrives at b_stall; report the time-out and leave
         __syncthreads();
         if (tid == 0 && !mbar_wait(b_stall, 0u, abort_flag, g.wait_ns)) atomicExch(g.err, TC_ERR_TIMEOUT);
