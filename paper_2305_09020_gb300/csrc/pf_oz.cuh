@@ -10,8 +10,8 @@
 //   X = sum_s x_s 256^(6-s), seven balanced digits -128 <= x_s <= 128, stored as FP16 integers.
 // X Y summed over k is sum_d 256^(12-d) v_d with the level sums v_d = sum_{s+t=d} sum_k x_s y_t.  Levels
 // 0..6 (28 digit products) are kept: the first dropped level is 2^-56 of a product of two row maxima.
-// Within a stage of 32 k every level sum is an integer below 7 * 32 * 2^14 < 2^22, so the tensor core's
-// FP32 accumulation is exact.  The drain adds v_d, in units of 256^7, into 64-bit integers:
+// Over a group of 128 k every level sum is an integer of at most 7 * 128 * 2^14 < 2^24, so the tensor core's
+// FP32 accumulation is exact.  The drain of a group adds v_d, in units of 256^7, into 64-bit integers:
 //   acc += v_0 2^40 + v_1 2^32 + v_2 2^24 + v_3 2^16 + v_4 2^8 + v_5 + rint(v_6 / 256),
 // which also is exact but for v_6 and stays below 2^63 for K < 512.  The result is rounded to double once.
 // Against FMA chains, whose rounding grows with K, the error is smaller.
@@ -32,15 +32,14 @@ namespace pf {
 constexpr int OZ_S = 7;                       // digits per operand
 constexpr int OZ_KC = 32;                     // K per stage: 64-byte rows of FP16
 constexpr int OZ_BM = 128;                    // rows per unit = TMEM lanes
-constexpr int OZ_MAXH = 24;                   // accumulator columns per drain thread: BN <= 96
+constexpr int OZ_MAXH = 16;                   // accumulator columns per drain thread: BN <= 64
+constexpr int OZ_GRP = 4;                     // stages per accumulation group (128 k)
 constexpr int OZ_MAXK = 480;                  // K bound of the 64-bit sums (< 512)
-constexpr int OZ_MAXR = 16;                   // TMEM regions in the ring at most
 constexpr int OZ_EPI_WARPS = 16;              // four warpgroups: a quarter of the columns each
 constexpr int OZ_THREADS = 640;
 // the launch holds 640 x 96 = 61440 registers: 512 x 104 + 128 x 64 = 61440
 constexpr int OZ_REG_EPI = 104, OZ_REG_AUX = 64;
 static_assert(512 * OZ_REG_EPI + 128 * OZ_REG_AUX <= OZ_THREADS * 96, "the setmaxnreg split must fit the launch's registers");
-constexpr unsigned long long OZ_BIAS = 0x4B400000ull;   // bits of 1.5 2^23
 constexpr uint32_t OZ_ABYTES = OZ_S * OZ_BM * OZ_KC * 2;   // A digits of a stage
 constexpr int OZ_OUTC = 4, OZ_OUTP = 5;       // columns and row pitch (doubles) of a drain warp's store block
 constexpr size_t OZ_OUTBYTES = (size_t)OZ_EPI_WARPS * 32 * OZ_OUTP * 8;
@@ -52,9 +51,8 @@ struct OzArgs {
     int ntn;                  // column tiles
     int BNlast;               // width of the last one (multiple of 32)
     int nst;                  // K stages
-    int nr;                   // TMEM regions (even, nr BN <= tmem_cols)
     int stages;               // shared-memory stages
-    int tmem_cols;
+    int tmem_cols;            // >= OZ_S BN: a region per level
     int nunits;               // row tiles x column tiles
     const int *E, *F;         // exponents of A's rows and B's columns
     // epilogue: row m = p R + r; store 0: C[m ldc + n]; store 1: C[(p N + n) ldr + r]
@@ -76,8 +74,8 @@ constexpr size_t OZ_SMEM = 227 * 1024;
 inline int oz_kpad(int k) { return (k + OZ_KC - 1) / OZ_KC * OZ_KC; }
 
 // sizes of the product of `rows` rows with an N x N matrix: column tiles, stages, shared memory.  Column
-// tiles: enough units for the chip, against the cycles of a unit: 56 MMAs a stage of 36 + BN/4 cycles and
-// about 2500 + 60 per column around them.
+// tiles: enough units for the chip, against the cycles of a unit: 56 MMAs a stage of 40 + BN/4 cycles and
+// about 6000 + 130 per column around them.
 inline OzArgs oz_plan(long long rows, int N, int sms, size_t *smem) {
     OzArgs a{};
     const int mt = (int)((rows + OZ_BM - 1) / OZ_BM);
@@ -87,12 +85,11 @@ inline OzArgs oz_plan(long long rows, int N, int sms, size_t *smem) {
     for (int nt = (N + 4 * OZ_MAXH - 1) / (4 * OZ_MAXH); nt <= (N + 31) / 32; ++nt) {
         const int bn = ((N + nt - 1) / nt + 31) / 32 * 32, tiles = (N + bn - 1) / bn;
         const double rounds = (double)(((long long)mt * tiles + sms - 1) / sms);
-        const double t = rounds * (a.nst * (56.0 * (36.0 + 0.25 * bn)) + 2500.0 + 60.0 * bn);
+        const double t = rounds * (a.nst * (56.0 * (40.0 + 0.25 * bn)) + 6000.0 + 130.0 * bn);
         if (a.BN == 0 || t < 0.98 * best) { best = t; a.BN = bn; a.ntn = tiles; }
     }
     a.BNlast = ((N - (a.ntn - 1) * a.BN) + 31) / 32 * 32;
     a.tmem_cols = 512;
-    a.nr = (OZ_MAXR < 512 / a.BN ? OZ_MAXR : 512 / a.BN) / 2 * 2;
     const size_t stage = OZ_ABYTES + (size_t)OZ_S * a.BN * OZ_KC * 2, fit = (OZ_SMEM - OZ_FIXED) / stage;
     a.stages = fit < 4 ? (int)fit : 4;
     a.nunits = mt * a.ntn;
@@ -282,12 +279,13 @@ __device__ __forceinline__ bool oz_frozen(const OzArgs &g, int mt) {
 
 // ---- the GEMM: persistent, warp-specialised; a CTA walks units of 128 rows x BN columns -------------
 //   warp 16     TMA: per 32-wide K stage the digits of A (32 x 128 x 7) and of B (32 x BN x 7), one 3D box each
-//   warps 17-18 issue the MMAs level by level (6 first; each level of a stage into a tensor-memory region
-//               of its own from a ring), the levels in turn between the two warps
+//   warps 17-18 issue the MMAs level by level (6 first), each level into a tensor-memory region of its own
+//               that it accumulates over a group of four stages: levels 6, 3, 2 by one warp, 5, 4, 1, 0 by
+//               the other, 28 MMAs of a stage each.  The drain of a level overlaps the group's later
+//               levels and the next group's first stage
 //   warps 0-15  drain the regions into the 64-bit integers, then convert and store (the epilogues of
 //               k_gemm).  Sixteen, because this code overflows the schedulers' instruction caches and its
-//               fetches are shared by a scheduler's warps: with eight a level took 950 cycles of drain
-//               against 400 of MMAs
+//               fetches are shared by a scheduler's warps
 // setmaxnreg moves registers from warps 16-19 to the drain warps.  Every mbarrier wait is bounded as in
 // pf_tc.cuh: on time-out the error word is set, copies and MMAs in flight finish (bounded), tensor memory
 // is freed and the kernel returns.
@@ -295,16 +293,16 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                                                                   const __grid_constant__ CUtensorMap tmB, OzArgs g) {
     extern __shared__ __align__(1024) unsigned char oz_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
-    const int S = g.stages, BN = g.BN, NR = g.nr;
+    const int S = g.stages, BN = g.BN;
     const uint32_t BSL = (uint32_t)BN * OZ_KC * 2;            // bytes of one digit of B
     const uint32_t STAGE = OZ_ABYTES + OZ_S * BSL;
     double *outb = (double *)(base + (size_t)S * STAGE);
     uint64_t *bars = (uint64_t *)((unsigned char *)outb + OZ_OUTBYTES);
-    // barriers: full[4] (a stage's digits landed), empty[4] (both issuers' MMAs done with it), rfull[16] /
-    // rempty[16] (a region's MMAs done / drained), fin[2]
-    const uint32_t b_full = smem_u32(bars), b_empty = b_full + 32, b_rfull = b_empty + 32, b_rempty = b_rfull + 8 * OZ_MAXR,
-                   b_fin = b_rempty + 8 * OZ_MAXR;
-    uint32_t *tslot = (uint32_t *)(bars + 8 + 2 * OZ_MAXR + 2);
+    // barriers: full[4] (a stage's digits landed), empty[4] (both issuers' MMAs done with it), rfull[7] /
+    // rempty[7] (a level's group done / drained), fin[2]
+    const uint32_t b_full = smem_u32(bars), b_empty = b_full + 32, b_rfull = b_empty + 32, b_rempty = b_rfull + 8 * OZ_S,
+                   b_fin = b_rempty + 8 * OZ_S;
+    uint32_t *tslot = (uint32_t *)(bars + 8 + 2 * OZ_S + 2);
     volatile int *abort_flag = (volatile int *)(tslot + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -313,7 +311,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
             mbar_init(b_full + 8 * s, 1);
             mbar_init(b_empty + 8 * s, 2);
         }
-        for (int r = 0; r < OZ_MAXR; ++r) {
+        for (int r = 0; r < OZ_S; ++r) {
             mbar_init(b_rfull + 8 * r, 1);
             mbar_init(b_rempty + 8 * r, OZ_EPI_WARPS);
         }
@@ -366,12 +364,11 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
             }
             __syncwarp();
         } else if (warp <= OZ_EPI_WARPS + 2) {
-            // ---- MMA issuers: whole warps, one elected lane (see pf_tc.cuh); issuer w takes every other
-            // level of the sequence (seven a stage), so each starts at its own region and skips one -----
+            // ---- MMA issuers: whole warps, one elected lane (see pf_tc.cuh) ---------------------------
             const int w = warp - (OZ_EPI_WARPS + 1);
             const uint32_t id_full = idesc_f16(OZ_BM, BN), id_last = idesc_f16(OZ_BM, g.BNlast);
-            int s = 0, r = w, turn = 0;
-            uint32_t ph = 0, rph = 0;
+            int s = 0;
+            uint32_t ph = 0, gph = 1;   // stage phase; phase of the regions' drained barriers
             bool ok = true;
             for (int u = blockIdx.x; u < g.nunits && ok; u += gridDim.x) {
                 const int mt = u / ntn, nt = u - mt * ntn;
@@ -383,29 +380,30 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                     const uint32_t sa = smem_u32(base + (size_t)s * STAGE);
                     const uint64_t da = sdesc_sw64(sa), db = sdesc_sw64(sa + OZ_ABYTES);
                     const bool two = g.K - c * OZ_KC > 16;   // the last stage may hold one 16-wide step only
+                    const bool first = (c & (OZ_GRP - 1)) == 0, last = (c & (OZ_GRP - 1)) == OZ_GRP - 1 || c == nst - 1;
 #pragma unroll
                     for (int d = OZ_S - 1; d >= 0; --d) {
-                        if (turn == w) {
-                            if (!mbar_wait_warp(b_rempty + 8 * r, rph ^ 1u, abort_flag, g.wait_ns)) { fail(); ok = false; break; }
+                        const bool mine = (d == 6 || d == 3 || d == 2) ? w == 0 : w == 1;
+                        if (!mine) continue;
+                        if (first) {
+                            if (!mbar_wait_warp(b_rempty + 8 * d, gph, abort_flag, g.wait_ns)) { fail(); ok = false; break; }
                             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                            const uint32_t t = tmem + (uint32_t)(r * BN);
-                            if (elect_one()) {
-#pragma unroll
-                                for (int x = 0; x <= d; ++x) {
-                                    const uint64_t a = da + (uint64_t)(x * ((OZ_BM * OZ_KC * 2) >> 4));
-                                    const uint64_t b = db + (uint64_t)((d - x) * (int)(BSL >> 4));
-                                    mma_f16(t, a, b, idesc, x ? 1u : 0u);
-                                    if (two) mma_f16(t, a + 2, b + 2, idesc, 1u);   // the next 16 k: 32 bytes further
-                                }
-                                mma_commit(b_rfull + 8 * r);
-                            }
-                            __syncwarp();
-                            r += 2;
-                            if (r >= NR) { r -= NR; rph ^= 1u; }
                         }
-                        turn ^= 1;
+                        const uint32_t t = tmem + (uint32_t)(d * BN);
+                        if (elect_one()) {
+#pragma unroll
+                            for (int x = 0; x <= d; ++x) {
+                                const uint64_t a = da + (uint64_t)(x * ((OZ_BM * OZ_KC * 2) >> 4));
+                                const uint64_t b = db + (uint64_t)((d - x) * (int)(BSL >> 4));
+                                mma_f16(t, a, b, idesc, (x || !first) ? 1u : 0u);
+                                if (two) mma_f16(t, a + 2, b + 2, idesc, 1u);   // the next 16 k: 32 bytes further
+                            }
+                            if (last) mma_commit(b_rfull + 8 * d);
+                        }
+                        __syncwarp();
                     }
                     if (!ok) break;
+                    if (last) gph ^= 1u;
                     if (elect_one()) mma_commit(b_empty + 8 * s);
                     __syncwarp();
                     if (++s == S) { s = 0; ph ^= 1u; }
@@ -421,61 +419,39 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
         // ---- drain, epilogue (warps 0-7) ------------------------------------------------------------------
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REG_EPI));
         const int quarter = warp & 3, half = warp >> 2;   // 32 rows; which quarter of the columns
-        // Sums of the levels plus OZ_BIAS each (below), modulo 2^64; they start at minus the biases of a
-        // unit's stages.  Code runs at about five cycles an instruction and warp here (pf_tc.cuh), so a
-        // value takes two: a packed FP32 addition that leaves the integer in the low bits, and one
-        // multiply-add into the 64-bit sum (converting and shifting took six: 900 cycles a level).
-        constexpr unsigned long long BIAS = OZ_BIAS;
-        constexpr unsigned long long BIASES = (BIAS >> 8) + BIAS + (BIAS << 8) + (BIAS << 16) + (BIAS << 24) + (BIAS << 32) + (BIAS << 40);
-        const unsigned long long acc0 = 0ull - (unsigned long long)nst * BIASES;
-        unsigned long long acc[OZ_MAXH];
+        long long acc[OZ_MAXH];
 #pragma unroll
-        for (int j = 0; j < OZ_MAXH; ++j) acc[j] = acc0;
-        int r = 0;
-        uint32_t rph = 0;
+        for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
+        uint32_t gph = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < g.nunits && (ok || !g.err); u += gridDim.x) {
             const int mt = u / ntn, nt = u - mt * ntn;
             if (oz_frozen(g, mt)) continue;
-            const int hbn = (nt == ntn - 1 ? g.BNlast : BN) >> 2;   // columns per thread (a multiple of 8)
+            const int hbn = (nt == ntn - 1 ? g.BNlast : BN) >> 2;   // columns per thread (8 or 16)
             const uint32_t lane0 = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * hbn);
-            for (int c = 0; c < nst && ok; ++c) {
+            for (int c = 0; c < nst && ok; c += OZ_GRP, gph ^= 1u) {
 #pragma unroll
                 for (int d = OZ_S - 1; d >= 0; --d) {
-                    if (!mbar_wait(b_rfull + 8 * r, rph, abort_flag, g.wait_ns)) { ok = false; break; }
+                    if (!mbar_wait(b_rfull + 8 * d, gph, abort_flag, g.wait_ns)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t ta = lane0 + (uint32_t)(r * BN);
-#pragma unroll
-                    for (int j0 = 0; j0 < OZ_MAXH; j0 += 8) {
-                        if (j0 < hbn) {
-                            float v[8];
-                            tmem_ld8(ta + (uint32_t)j0, v);
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                            for (int j = 0; j < 8; j += 2) {
-                                // v is an integer below 2^22: the bits of v + 1.5 2^23 are OZ_BIAS + v (level 6:
-                                // + 128 more, so that its shift by 8 rounds)
-                                const float mg = d == 6 ? 12582912.f + 128.f : 12582912.f;
-                                unsigned long long x, y, z;
-                                asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(v[j]), "f"(v[j + 1]));
-                                asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(mg));
-                                asm("add.rn.f32x2 %0, %1, %2;" : "=l"(z) : "l"(x), "l"(y));
-                                const unsigned int w0 = (unsigned int)z, w1 = (unsigned int)(z >> 32);
-                                unsigned long long &a0 = acc[j0 + j], &a1 = acc[j0 + j + 1];
-                                if (d == 6) {
-                                    a0 += (unsigned long long)(w0 >> 8);
-                                    a1 += (unsigned long long)(w1 >> 8);
-                                } else {
-                                    a0 += (unsigned long long)w0 << (8 * (5 - d));
-                                    a1 += (unsigned long long)w1 << (8 * (5 - d));
-                                }
-                            }
-                        }
-                    }
+                    const uint32_t ta = lane0 + (uint32_t)(d * BN);
+                    float v[OZ_MAXH];
+                    tmem_ld8(ta, v);
+                    if (hbn > 8) tmem_ld8(ta + 8u, v + 8);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(b_rempty + 8 * r);
-                    if (++r == NR) { r = 0; rph ^= 1u; }
+                    if (lane == 0) mbar_arrive(b_rempty + 8 * d);
+#pragma unroll
+                    for (int j0 = 0; j0 < OZ_MAXH; j0 += 8)
+                        if (j0 < hbn) {
+#pragma unroll
+                            for (int j = j0; j < j0 + 8; ++j) {
+                                const int w = __float2int_rn(v[j]);   // an integer
+                                if (d == 6) acc[j] += (long long)((w + 128) >> 8);
+                                else acc[j] += (long long)w * (1ll << (8 * (5 - d)));
+                            }
+                        }
                 }
             }
             if (!ok) {
@@ -518,7 +494,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                 }
 #pragma unroll
                 for (int j = 0; j < OZ_OUTC; ++j) {   // units 2^56 of X Y 2^(E + F - 2154)
-                    v[j] = oz_double((long long)acc[j], em + __shfl_sync(0xffffffffu, fl, j0 + j) - 2154 + 56);
+                    v[j] = oz_double(acc[j], em + __shfl_sync(0xffffffffu, fl, j0 + j) - 2154 + 56);
                     if (nan) v[j] = __longlong_as_double(0x7FF8000000000000ll);
                 }
                 if (g.store == 1) {             // lanes hold consecutive rows: coalesced as it is
@@ -571,7 +547,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                 for (int j = 0; j + OZ_OUTC < OZ_MAXH; ++j) acc[j] = acc[j + OZ_OUTC];
             }
 #pragma unroll
-            for (int j = 0; j < OZ_MAXH; ++j) acc[j] = acc0;
+            for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
