@@ -559,11 +559,9 @@ struct Engine {
             // reciprocals for the solves of the steady step (the others divide)
             const int j = s.bdf == 2 ? 1 : 0;
             add_rcp(PF_BCSET_V, shV);
-            if (s.precision == PF_FP64) {   // a mixed run's FP64 engine only finds the initial potential
-                add_rcp(PF_BCSET_NN, shPsi[j]);
-                add_rcp(PF_BCSET_NN, shPhi[j]);
-            }
-            if (s.precision == PF_FP64 && s.model != PF_MODEL_EQUILIBRIUM) {
+            add_rcp(PF_BCSET_NN, shPsi[j]);
+            add_rcp(PF_BCSET_NN, shPhi[j]);
+            if (s.model != PF_MODEL_EQUILIBRIUM) {
                 add_rcp(PF_BCSET_P, shP);
                 add_rcp(PF_BCSET_U, shU[j]);
             }
@@ -576,8 +574,11 @@ struct Engine {
     // Eight launches a solve of about 5 us at least against the SIMT transforms' three or four: measured
     // per 2D step, 24 x 13 nodes 0.277 / 0.271 ms (digits / SIMT), 30 x 16 0.279 / 0.289, 48 x 25 0.310 /
     // 0.384, 240 x 121 0.571 / 1.276
+    // The FP64 engine that only finds a mixed run's initial potential keeps the FMA transforms: a last bit
+    // of V^0 moves the FP32 rounding of every later step (P by 1e-5 after four steps).
     bool oz_pays() const {
-        return std::max(nx, ny) >= 28 && nx <= pf::OZ_MAXK && ny <= pf::OZ_MAXK && tc_encode() != nullptr;
+        return hs.precision == PF_FP64 && std::max(nx, ny) >= 28 && nx <= pf::OZ_MAXK && ny <= pf::OZ_MAXK &&
+               tc_encode() != nullptr;
     }
     // digits and exponents of Bt's rows (Bt n x n row-major: B's columns)
     void add_oz(const T *key, const std::vector<double> &Bt, int n) {
