@@ -1130,28 +1130,52 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 2) k_fwd(Geo<T> G, F
         for (int c = 0; c < 4; ++c) ssrc[ql * 4 + c] = s[c];
     }
     pdl_enter();   // the twiddles and sources above are constants of the run
-    __syncthreads();
+    int corner = 0;    // does the block hold a node of four elements?
+    for (int ql = threadIdx.x; ql < tp; ql += blockDim.x) corner |= ssrc[ql * 4 + 2] >= 0;
+    corner = __syncthreads_or(corner);
     const long long lplane = (long long)G.ex * G.ey * G.p * G.p;
     const int lgtp = 31 - __clz(tp);          // tp is a power of two dividing blockDim.x
     {
-        // this thread's pencil column is fixed (blockDim.x is a multiple of tp): its DSSUM sources
-        // live in registers, and it walks the planes z0, z0 + zs, ... eight gathers at a time
+        // this thread's pencil column is fixed (blockDim.x is a multiple of tp): its DSSUM sources live in
+        // registers, and it walks the planes z0, z0 + zs, ... several gathers at a time.  A node has one
+        // or two sources but for the corners: both are loaded by every thread, without a branch that
+        // would keep the next plane's loads from starting (a missing one repeats the first and is not
+        // added)
         const int ql = threadIdx.x & (tp - 1), qg = q0 + ql, z0 = threadIdx.x >> lgtp, zs = blockDim.x >> lgtp;
         int sr[4];
+        bool has[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) sr[c] = ssrc[ql * 4 + c];
+        for (int c = 0; c < 4; ++c) {
+            sr[c] = ssrc[ql * 4 + c];
+            has[c] = sr[c] >= 0;
+        }
+#pragma unroll
+        for (int c = 3; c >= 0; --c)
+            if (!has[c]) sr[c] = max(sr[0], 0);
         const bool live = qg < G.n2;
-        for (int zb = z0; zb < nz; zb += 8 * zs) {
-            T v0[8], v1[8];
+        auto gather = [&](const T *__restrict__ L, int z) {
+            const T *p = L + z * lplane;
+            const T x0 = p[sr[0]], x1 = p[sr[1]];
+            T v = has[1] ? x0 + x1 : x0;
+            if (corner) {
+                const T x2 = p[sr[2]], x3 = p[sr[3]];
+                if (has[2]) v += x2;
+                if (has[3]) v += x3;
+            }
+            return v;
+        };
+        constexpr int U = 4;
+        for (int zb = z0; zb < nz; zb += U * zs) {
+            T v0[U], v1[U];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {   // eight independent gathers in flight
-                const int z = zb + u * zs;
-                v0[u] = 0;
+            for (int u = 0; u < U; ++u) {   // independent gathers in flight
+                const int z = min(zb + u * zs, nz - 1);
                 v1[u] = 0;
-                if (live && z < nz) {
-                    const long long gi = (long long)z * G.n2 + qg;
-                    v0[u] = a.x0_local ? gather4(a.X0, z * lplane, sr) : a.X0[gi];
-                    if (a.X1) v1[u] = a.x1_local ? gather4(a.X1, z * lplane, sr) : a.X1[gi];
+                if (a.x0_local) v0[u] = gather(a.X0, z);
+                else v0[u] = live ? a.X0[(long long)z * G.n2 + qg] : T(0);
+                if (a.X1) {
+                    if (a.x1_local) v1[u] = gather(a.X1, z);
+                    else v1[u] = live ? a.X1[(long long)z * G.n2 + qg] : T(0);
                 }
             }
 #pragma unroll
