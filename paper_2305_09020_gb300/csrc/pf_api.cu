@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdint>
 #include <cstring>
 #include <memory>
 #include <string>
@@ -1862,6 +1863,37 @@ extern "C" int pf_sync(pf_handle *h) {
 }
 
 namespace {
+// the device's address of n doubles at host address p, or null unless one pinned allocation that kernels may
+// write holds all of them (not pageable, misaligned, read-only or I/O memory, nor two pinned pieces with a gap)
+double *pinned_span(double *p, size_t n) {
+    using GetAttr = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+    static const GetAttr get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<GetAttr>(f);
+    }();
+    cudaPointerAttributes at{};
+    unsigned flags = 0;
+    if (!get || reinterpret_cast<std::uintptr_t>(p) % alignof(double) || cudaPointerGetAttributes(&at, p) != cudaSuccess || at.type != cudaMemoryTypeHost || !at.devicePointer ||
+        cudaHostGetFlags(&flags, p) != cudaSuccess || (flags & ~(cudaHostAllocPortable | cudaHostAllocMapped))) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const CUdeviceptr d = reinterpret_cast<CUdeviceptr>(at.devicePointer);
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    if (get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, d) != CUDA_SUCCESS ||
+        get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, d) != CUDA_SUCCESS)
+        return nullptr;
+    return d >= start && d - start <= size && n * sizeof(double) <= size - (d - start) ? static_cast<double *>(at.devicePointer)
+                                                                                       : nullptr;
+}
+
 template <typename T>
 int get_impl(pf_handle *h, Engine<T> &E, unsigned mask, double *out, size_t n) {
     const bool old = mask & PF_FIELD_OLD;
@@ -1874,6 +1906,24 @@ int get_impl(pf_handle *h, Engine<T> &E, unsigned mask, double *out, size_t n) {
     if (mask & PF_FIELD_P) need += 1;
     if (mask & PF_FIELD_U) need += 3;
     if (need * (size_t)E.N > n) return fail(h, PF_EINVAL, "output buffer too small");
+    // pinned memory: one kernel stores every field there (psi, which is formed on the host, goes the long way)
+    double *dev_out = need > 0 && !(mask & PF_FIELD_PSI) ? pinned_span(out, need * E.N) : nullptr;
+    if (dev_out) {
+        pf::FieldsOut<T> f{};
+        auto add = [&](const T *src) { f.src[f.n++] = src; };
+        if (mask & PF_FIELD_V) add(E.V[l]);
+        if (mask & PF_FIELD_E) { add(E.Ex); add(E.Ey); add(E.d3 ? E.Ez[E.cur] : nullptr); }
+        if (mask & PF_FIELD_PHI) add(E.phi[l]);
+        if (mask & PF_FIELD_P) add(E.P[l]);
+        if (mask & PF_FIELD_U) { add(E.u[0][l]); add(E.u[1][l]); add(E.u[2][l]); }
+        const unsigned blocks = (unsigned)std::min<long long>((E.N + 255) / 256, 304);
+        E.prof->begin(PF_KC_OTHER, E.st);
+        pf::k_fields_out<T><<<dim3(blocks, f.n), 256, 0, E.st>>>(f, E.N, dev_out);
+        E.check_launch();
+        E.prof->end(E.st);
+        PF_CU(cudaStreamSynchronize(E.st));
+        return PF_OK;
+    }
     PF_CU(cudaStreamSynchronize(E.st));
     double *o = out;
     auto put = [&](const T *src) {

@@ -1179,7 +1179,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 2) k_fwd(Geo<T> G, F
                 }
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int z = zb + u * zs;
                 if (z < nz) buf[ql * ld + fft_slot(z, bits, pow2)] = {v0[u], v1[u]};
             }
@@ -2465,6 +2465,22 @@ __global__ void k_energy(Geo<T> G, EnergyConst c, const T *__restrict__ phi, con
         for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
         part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
     }
+}
+
+// up to ten fields of n values as FP64 blocks in mapped (pinned) host memory, zeros for a null source: the
+// conversion and the way over the link in one launch for all fields (a conversion into scratch and a copy
+// per field: two launches each, and the link idle during the conversions)
+template <typename T>
+struct FieldsOut {
+    const T *src[10];
+    int n;
+};
+template <typename T>
+__global__ void k_fields_out(FieldsOut<T> f, long long n, double *__restrict__ out) {
+    const T *src = f.src[blockIdx.y];
+    out += (long long)blockIdx.y * n;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = src ? (double)src[i] : 0.0;
 }
 
 template <typename T, typename S>
