@@ -242,9 +242,6 @@ def warmstart_arm(args):
     return 0
 
 
-# pinned FP64 transform variant per workload (what the autotuner picks on the GB300): cp.async 32x32
-# tiles with the fused y pair
-FP64_VARIANT = (4, 1)
 # timed oracle steps of the CPU baseline per workload (about 10-30 s of host work)
 ORACLE_STEPS = {"layers3d": 10, "droplet3d": 10, "electrode_array3d": 5, "patches2d": 10}
 
@@ -260,7 +257,6 @@ def fp64_leg(args, wl, dof, prec, gemm_choice, fused_y, fft_tile, stream, flush,
     ALL_FIELDS = (native.PF_FIELD_V | native.PF_FIELD_E | native.PF_FIELD_PHI | native.PF_FIELD_PSI |
                   native.PF_FIELD_P | native.PF_FIELD_U)
     h64 = native.from_workload(wl, precision=native.PF_FP64, stream=stream.cuda_stream)
-    h64.set_variant(*FP64_VARIANT)
     hm = native.from_workload(wl, precision=prec, stream=stream.cuda_stream)
     hm.set_variant(gemm_choice, fuse_y=bool(fused_y), tile=fft_tile)
     n = max(1, args.err_steps)
@@ -286,7 +282,7 @@ def fp64_leg(args, wl, dof, prec, gemm_choice, fused_y, fft_tile, stream, flush,
     ms64 = sum(a.elapsed_time(b) for a, b in ev) / k64
     h64.close()
     return {"value": dof / (ms64 * 1e-3), "unit": UNIT, "ms_per_step": ms64, "steps": k64,
-            "variant": transform_kernel(*FP64_VARIANT) + " (FP64, pinned)",
+            "variant": "k_oz_split + k_gemm_oz (FP64 default: exact digit products on the tensor cores)",
             "err_steps": n,
             "mixed_rel_l2_vs_fp64": err,
             "note": "relative L2 per field of the mixed path against the FP64 GPU path after err_steps steps "
