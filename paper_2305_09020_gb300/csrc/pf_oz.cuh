@@ -16,8 +16,8 @@
 // which also is exact but for v_6 and stays below 2^63 for K < 512.  The result is rounded to double once.
 // Against FMA chains, whose rounding grows with K, the error is smaller.
 //
-// A row with an infinity or NaN gives NaN results; other rows are not affected.  Subnormal entries keep
-// their bits; results are rounded to nearest, ties to even.
+// A row of A or a column of B with an infinity or NaN gives NaN results; other rows and columns are not
+// affected.  Subnormal entries keep their bits; results are rounded to nearest, ties to even.
 #pragma once
 
 #include <cuda.h>
@@ -483,8 +483,9 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                 }
 #pragma unroll
                 for (int j = 0; j < OZ_OUTC; ++j) {   // units 2^56 of X Y 2^(E + F - 2154)
-                    v[j] = oz_double(acc[j], em + __shfl_sync(0xffffffffu, fl, j0 + j) - 2154 + 56);
-                    if (nan) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+                    const int fn = __shfl_sync(0xffffffffu, fl, j0 + j);
+                    v[j] = oz_double(acc[j], em + fn - 2154 + 56);
+                    if (nan || fn == 0x7FF) v[j] = __longlong_as_double(0x7FF8000000000000ll);
                 }
                 if (g.store == 1) {             // lanes hold consecutive rows: coalesced as it is
 #pragma unroll
