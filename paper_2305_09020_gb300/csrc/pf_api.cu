@@ -262,7 +262,7 @@ struct Engine {
     struct OzB {
         const T *key;
         __half *dig;      // [OZ_S][n][Kpad]
-        int *F;
+        int *F, *sh;      // exponents of the columns, shifts of the rows
         int n, Kpad;
     };
     std::vector<OzB> ozb;
@@ -581,35 +581,37 @@ struct Engine {
         return hs.precision == PF_FP64 && std::max(nx, ny) >= 28 && nx <= pf::OZ_MAXK && ny <= pf::OZ_MAXK &&
                tc_encode() != nullptr;
     }
-    // digits and exponents of Bt's rows (Bt n x n row-major: B's columns)
+    // digits and exponents of Bt's rows (Bt n x n row-major: B's columns), balanced by the shifts of B's rows
     void add_oz(const T *key, const std::vector<double> &Bt, int n) {
         OzB t;
         t.key = key;
         t.n = n;
         t.Kpad = oz_kpad(n);
         std::vector<__half> dig((size_t)pf::OZ_S * n * t.Kpad, __float2half(0.f));
-        std::vector<int> F(n);
+        std::vector<int> F(n), sh(t.Kpad, pf::OZ_SKIP);
+        auto bits = [&](int r, int k) {
+            unsigned long long u;
+            std::memcpy(&u, &Bt[(size_t)r * n + k], 8);
+            return u;
+        };
+        for (int r = 0; r < n; ++r)
+            for (int k = 0; k < n; ++k) sh[k] = std::max(sh[k], pf::oz_exp(bits(r, k), -1023));
         for (int r = 0; r < n; ++r) {
-            auto bits = [&](int k) {
-                unsigned long long u;
-                std::memcpy(&u, &Bt[(size_t)r * n + k], 8);
-                return u;
-            };
-            int em = 1;
-            for (int k = 0; k < n; ++k) em = std::max(em, (int)(bits(k) >> 52) & 0x7FF);
+            int em = pf::OZ_SKIP;
+            for (int k = 0; k < n; ++k) em = std::max(em, pf::oz_exp(bits(r, k), -sh[k]));
             F[r] = em;
             for (int k = 0; k < n; ++k) {
-                const unsigned long long u = pf::oz_fixed(bits(k), em);
-                for (int d = 0; d < pf::OZ_S; ++d) {
-                    const int v = d == 0 ? (int)(u >> 48) - 128 : (int)((u >> (8 * (6 - d))) & 0xFF) - 128;
-                    dig[((size_t)d * n + r) * t.Kpad + k] = __float2half((float)v);
-                }
+                const unsigned long long u = pf::oz_fixed(bits(r, k), em - pf::oz_exp(bits(r, k), -sh[k]));
+                for (int d = 0; d < pf::OZ_S; ++d)
+                    dig[((size_t)d * n + r) * t.Kpad + k] = __float2half((float)((int)((u >> (8 * (7 - d))) & 0xFF) - 128));
             }
         }
         t.dig = mk<__half>(dig.size());
         t.F = mk<int>(n);
+        t.sh = mk<int>(t.Kpad);
         PF_CU(cudaMemcpyAsync(t.dig, dig.data(), dig.size() * sizeof(__half), cudaMemcpyHostToDevice, st));
         PF_CU(cudaMemcpyAsync(t.F, F.data(), n * sizeof(int), cudaMemcpyHostToDevice, st));
+        PF_CU(cudaMemcpyAsync(t.sh, sh.data(), t.Kpad * sizeof(int), cudaMemcpyHostToDevice, st));
         PF_CU(cudaStreamSynchronize(st));
         ozb.push_back(t);
     }
@@ -621,7 +623,7 @@ struct Engine {
         check_launch();
         ozrcp.push_back({bcset, sh, q});
     }
-    // digit planes [OZ_S][rows][Kpad], boxes of 32 x box x 7
+    // digit planes [OZ_S][rows][Kpad], boxes of 32 x box x 8
     CUtensorMap ozmap(const __half *ptr, long long rows, int Kpad, int box_rows) {
         for (auto &m : ozmaps)
             if (m.ptr == ptr && m.rows == rows && m.Kpad == Kpad && m.box == box_rows) return m.map;
@@ -655,7 +657,7 @@ struct Engine {
         const CUtensorMap ma = ozmap(ozdig, rows, ob->Kpad, pf::OZ_BM), mb = ozmap(ob->dig, N, ob->Kpad, a.BN);
         const double *A64 = reinterpret_cast<const double *>(A);
         prof->begin(PF_KC_GEMM, st);
-        pf::oz_split(A64, N, 1, a.M, N, ozdig, ozE, R, active, nz, st, pdl());
+        pf::oz_split(A64, a.M, N, ob->sh, ozdig, ozE, R, active, nz, st, pdl());
         check_launch();
         prof->end(st);
         prof->begin(PF_KC_GEMM, st);

@@ -1579,6 +1579,7 @@ struct GemmArgs {
     const T *m2x, *m2y, *face2;
     const int *active;   // ensembles: per-run flags (0 = frozen), run = plane % amod; null otherwise
     int amod;
+    const int *only_if;  // nullable: k_gemm does nothing where it holds 0
 };
 
 // ensembles: true when every row of the tile [m0, m0 + BM) belongs to a frozen run (plane = m / R)
@@ -1593,6 +1594,7 @@ __device__ __forceinline__ bool tile_frozen(const GemmArgs<T> &g, long long m0, 
 
 template <typename T, int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm(GemmArgs<T> g) {
+    if (g.only_if && !*g.only_if) return;
     if (tile_frozen(g, (long long)blockIdx.y * BM, BM)) return;
     constexpr int NTH = (BM / TM) * (BN / TN);
     constexpr int LA = BM * BK / NTH;   // A elements staged per thread per k tile

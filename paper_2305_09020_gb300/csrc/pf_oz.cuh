@@ -3,21 +3,37 @@
 // C[M x N] = A[M x K] * B[K x N] for the constant eigenbasis products of the Remark after Algorithm 2 in
 // double precision.  The FP64 pipe of the GB300 runs 2 FMA per SM and cycle (1.1 TFLOP/s measured), the
 // tensor cores 4096 FP16 products, and small integers multiply and add exactly there.  So each operand
-// is written in fixed point (the integer splitting of Ozaki, Ogita, Oishi and Rump for matrix units):
-//   row m of A:     a = X 2^(E_m - 1077),  X = rint(a 2^(1077 - E_m)), |X| < 2^55,
-//                   E_m the largest biased exponent of the row,
-//   column n of B:  b = Y 2^(F_n - 1077), the same (split once on the host),
-//   X = sum_s x_s 256^(6-s), seven balanced digits -128 <= x_s <= 128, stored as FP16 integers.
-// X Y summed over k is sum_d 256^(12-d) v_d with the level sums v_d = sum_{s+t=d} sum_k x_s y_t.  Levels
-// 0..6 (28 digit products) are kept: the first dropped level is 2^-56 of a product of two row maxima.
-// Over a group of 128 k every level sum is an integer of at most 7 * 128 * 2^14 < 2^24, so the tensor core's
-// FP32 accumulation is exact.  The drain of a group adds v_d, in units of 256^7, into 64-bit integers:
-//   acc += v_0 2^40 + v_1 2^32 + v_2 2^24 + v_3 2^16 + v_4 2^8 + v_5 + rint(v_6 / 256),
-// which also is exact but for v_6 and stays below 2^63 for K < 512.  The result is rounded to double once.
-// Against FMA chains, whose rounding grows with K, the error is smaller.
+// is written in fixed point (the integer splitting of Ozaki, Ogita, Oishi and Rump for matrix units), after
+// the terms a_mk b_kn of a sum have been balanced by an exact power of two per k:
+//   s_k             the largest biased exponent of B's row k less 1023 (a table of the basis; rows of zeros,
+//                   the eigenbases' constrained nodes, are left out of A whatever A holds there),
+//   row m of A:     a_mk 2^s_k = X 2^(E_m - 1084),  X = rint(a_mk 2^(s_k + 1084 - E_m)), |X| < 2^62,
+//                   E_m the largest biased exponent of the balanced row,
+//   column n of B:  b_kn 2^-s_k = Y 2^(F_n - 1084), the same,
+//   X = sum_s x_s 256^(7-s), eight balanced digits -128 <= x_s <= 127 (|x_0| <= 64), stored as FP16 integers.
+// X Y summed over k is sum_d 256^(14-d) v_d with the level sums v_d = sum_{s+t=d} sum_k x_s y_t.  Levels
+// 0..7 (36 digit products) are kept: the first dropped level is about 2^-61 of the product of the largest
+// balanced entries of row and column.  Over a group of 128 k every level sum is an integer of at most
+// 128 (6 2^14 + 2 2^13) < 2^24, so the tensor core's FP32 accumulation is exact.  The drain of a group adds the
+// levels into a 64-bit integer and a byte of fraction, in units of 256^8:
+//   256 acc + frac += v_0 2^48 + v_1 2^40 + v_2 2^32 + v_3 2^24 + v_4 2^16 + v_5 2^8 + v_6 + rint(v_7 / 256),
+// which is exact but for v_7; |acc| < 2^62 for K < 512.  The result is rounded to double once.
+//
+// The error is relative to the largest balanced entries, an FMA chain's to the sum of the terms' sizes.
+// Balanced, the largest entry of A meets an entry of its own size in B's row, so that the row of C holds a value
+// as large as that product, and eight digits leave 2^-61 of it where a chain leaves 2^-53 per term: no plane, row
+// or column of a solve is further off than with the chains (tests: even, cosine and geometric meshes to a ratio
+// of 4^10 in size, values of 1e200 at constrained nodes).  Measured against extended precision, 105 x 43
+// nodes on a cosine mesh, plane / worst row / worst column: chains 8.4e-16 / 1.3e-15 / 2.9e-15, seven digits
+// without the balance 1.1e-15 / 6.1e-14 / 5.7e-15 (and no digit left for a value of 1e16 at a constrained node),
+// seven with it 6e-16 / 1.6e-14 / 4e-15, these 1.2e-16 /
+// 2.0e-16 / 3.0e-16.
+// What cannot be balanced per k is a basis of uncoupled pieces (zeros inside rows and columns that are not
+// zero): entries of one piece would take digits from another.  The allocation-free solve, whose bases are the
+// caller's, finds those on the device and takes the FMA kernels (pf_static.cu); a run's own have none.
 //
 // A row of A or a column of B with an infinity or NaN gives NaN results; other rows and columns are not
-// affected.  Subnormal entries keep their bits; results are rounded to nearest, ties to even.
+// affected.  Subnormal entries keep their bits; normal results are rounded to nearest, ties to even.
 #pragma once
 
 #include <cuda.h>
@@ -29,19 +45,21 @@
 
 namespace pf {
 
-constexpr int OZ_S = 7;                       // digits per operand
+constexpr int OZ_S = 8;                       // digits per operand, levels of the product
 constexpr int OZ_KC = 32;                     // K per stage: 64-byte rows of FP16
 constexpr int OZ_BM = 128;                    // rows per unit = TMEM lanes
 constexpr int OZ_MAXH = 16;                   // accumulator columns per drain thread: BN <= 64
 constexpr int OZ_GRP = 4;                     // stages per accumulation group (128 k)
 constexpr int OZ_MAXK = 480;                  // K bound of the 64-bit sums (< 512)
+constexpr int OZ_SKIP = -(1 << 20);           // shift of a k whose row of B is zero
+constexpr int OZ_NONFINITE = 1 << 20;         // exponent of a row or column with an infinity or NaN
 constexpr int OZ_EPI_WARPS = 16;              // four warpgroups: a quarter of the columns each
 constexpr int OZ_THREADS = 640;
 // the launch holds 640 x 96 = 61440 registers: 512 x 104 + 128 x 64 = 61440
 constexpr int OZ_REG_EPI = 104, OZ_REG_AUX = 64;
 static_assert(512 * OZ_REG_EPI + 128 * OZ_REG_AUX <= OZ_THREADS * 96, "the setmaxnreg split must fit the launch's registers");
 constexpr uint32_t OZ_ABYTES = OZ_S * OZ_BM * OZ_KC * 2;   // A digits of a stage
-constexpr int OZ_OUTC = 4, OZ_OUTP = 5;       // columns and row pitch (doubles) of a drain warp's store block
+constexpr int OZ_OUTC = 4, OZ_OUTP = 5;       // columns (a word of fractions) and row pitch (doubles) of a drain warp's store block
 constexpr size_t OZ_OUTBYTES = (size_t)OZ_EPI_WARPS * 32 * OZ_OUTP * 8;
 constexpr size_t OZ_FIXED = 1024 + OZ_OUTBYTES + 512;      // alignment slack; store blocks; barriers, TMEM slot
 
@@ -66,15 +84,16 @@ struct OzArgs {
     const double *m2x, *m2y, *face2;
     const int *active;        // ensembles: per-run flags (0 = frozen), run = p % amod; null otherwise
     int amod;
+    const int *skip_if;       // nullable: nothing is done where it holds a value that is not 0
     int *err;                 // error word; null: a call without one, whose results become NaN on a time-out
     unsigned long long wait_ns;
 };
 
 constexpr size_t OZ_SMEM = 227 * 1024;
-inline int oz_kpad(int k) { return (k + OZ_KC - 1) / OZ_KC * OZ_KC; }
+__host__ __device__ inline int oz_kpad(int k) { return (k + OZ_KC - 1) / OZ_KC * OZ_KC; }
 
 // sizes of the product of `rows` rows with an N x N matrix: column tiles, stages, shared memory.  Column
-// tiles: enough units for the chip, against the cycles of a unit: 56 MMAs a stage of 40 + BN/4 cycles and
+// tiles: enough units for the chip, against the cycles of a unit: 72 MMAs a stage of 40 + BN/4 cycles and
 // about 6000 + 130 per column around them.
 inline OzArgs oz_plan(long long rows, int N, int sms, size_t *smem) {
     OzArgs a{};
@@ -85,7 +104,7 @@ inline OzArgs oz_plan(long long rows, int N, int sms, size_t *smem) {
     for (int nt = (N + 4 * OZ_MAXH - 1) / (4 * OZ_MAXH); nt <= (N + 31) / 32; ++nt) {
         const int bn = ((N + nt - 1) / nt + 31) / 32 * 32, tiles = (N + bn - 1) / bn;
         const double rounds = (double)(((long long)mt * tiles + sms - 1) / sms);
-        const double t = rounds * (a.nst * (56.0 * (40.0 + 0.25 * bn)) + 6000.0 + 130.0 * bn);
+        const double t = rounds * (a.nst * (72.0 * (40.0 + 0.25 * bn)) + 6000.0 + 130.0 * bn);
         if (a.BN == 0 || t < 0.98 * best) { best = t; a.BN = bn; a.ntn = tiles; }
     }
     a.BNlast = ((N - (a.ntn - 1) * a.BN) + 31) / 32 * 32;
@@ -97,7 +116,7 @@ inline OzArgs oz_plan(long long rows, int N, int sms, size_t *smem) {
     return a;
 }
 
-// digit planes [OZ_S][rows][Kpad], boxes of 32 x box_rows x 7
+// digit planes [OZ_S][rows][Kpad], boxes of 32 x box_rows x 8
 inline bool oz_encode(CUtensorMap *m, const __half *ptr, long long rows, int Kpad, int box_rows) {
     cuuint64_t dims[3] = {(cuuint64_t)Kpad, (cuuint64_t)rows, (cuuint64_t)OZ_S};
     cuuint64_t strides[2] = {(cuuint64_t)Kpad * 2, (cuuint64_t)Kpad * 2 * rows};
@@ -141,22 +160,29 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-// biased fixed point of a against the row exponent emax (>= a's): X + 128 (256^6 + .. + 1), so that byte s
-// from the top (16 bits for s = 0) is digit x_s + 128
-__host__ __device__ __forceinline__ unsigned long long oz_fixed(unsigned long long bits, int emax) {
-    const int e = (int)(bits >> 52) & 0x7FF;
+// biased fixed point of a double whose balanced exponent lies r >= 0 below its row's:
+// X + 128 (256^7 + .. + 1), so that byte s from the top is digit x_s + 128
+__host__ __device__ __forceinline__ unsigned long long oz_fixed(unsigned long long bits, int r) {
     unsigned long long m = bits & 0xFFFFFFFFFFFFFull;
-    if (e) m |= 1ull << 52;
-    int r = emax - (e ? e : 1);
-    if (r > 60) r = 60;
-    m = (((m << 3) >> r) + 1) >> 1;
+    if ((bits >> 52) & 0x7FF) m |= 1ull << 52;
+    if (r > 63) r = 63;
+    m = (((m << 10) >> r) + 1) >> 1;
     const unsigned long long s = 0ull - (bits >> 63);
-    return ((m ^ s) - s) + 0x0080808080808080ull;
+    return ((m ^ s) - s) + 0x8080808080808080ull;
+}
+// biased exponent of a double for oz_fixed (1 for subnormals), shifted; OZ_SKIP and less for 0 and a left-out k
+__host__ __device__ __forceinline__ int oz_exp(unsigned long long bits, int sh) {
+    const int e = (int)(bits >> 52) & 0x7FF;
+    return (bits << 1) ? (e ? e : 1) + sh : 2 * OZ_SKIP;
 }
 
-// v 2^sc rounded to nearest even: one conversion, the power of two added to its exponent (normalising by
-// integer operations instead took about thirty: 1 to 3% of a step)
-__device__ __forceinline__ double oz_double(long long v, int sc) {
+// (acc 256 + frac) 2^sc rounded to nearest even: one conversion (a rounding to odd keeps what does not fit into
+// 64 bits), the power of two added to its exponent.  Normalising by integer operations instead took
+// about thirty: 1 to 3% of a step
+__device__ __forceinline__ double oz_double(long long acc, int frac, int sc) {
+    const bool fits = (unsigned long long)(acc + (1ll << 54)) < (1ull << 55);
+    const long long v = fits ? acc * 256 + frac : (acc + (frac >> 8)) | ((frac & 0xFF) != 0);
+    if (!fits) sc += 8;
     const double x = __ll2double_rn(v);
     const int hi = __double2hiint(x), e = ((hi >> 20) & 0x7FF) + sc;
     if (v == 0) return 0.0;
@@ -170,19 +196,16 @@ __device__ __forceinline__ double oz_double(long long v, int sc) {
 
 #ifndef PF_OZ_HELPERS_ONLY
 // ---- digits of A: one warp per row ----------------------------------------------------------------
-// dig[d][m][Kpad] (FP16), E[m], of the rows A[m rs + k ks].  Bound by its 8 bytes read and 14 written per value, most of them in L2;
-// a pass of its own because inside the GEMM every column tile would split the rows again (measured there:
-// 7,000 issue slots per 128 x 32 stage against 3,100 cycles of MMAs).  NI = ceil(Kpad / 64) pairs a lane.
+// dig[d][m][Kpad] (FP16), E[m], of the values row[k ks] 2^(sg sh[k]) of row m.  NI = ceil(Kpad / 64) pairs a lane;
+// sh holds Kpad shifts.  sparse (nullable) is set where a row that is not zero has a zero at a k that is not
+// left out.
 template <int NI>
-__global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, long long rs, int ks, int M, int K, int Kpad,
-                                                  __half *__restrict__ dig, int *__restrict__ E, int R, const int *__restrict__ active, int amod) {
-    const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    tc_pdl_enter();
-    if (m >= M) return;
-    if (active && !active[(m / R) % amod]) return;   // a frozen run's rows: their products are not used
-    const double *row = A + m * rs;
+__device__ __forceinline__ void oz_split_row(const double *__restrict__ row, int ks, const int *__restrict__ sh, int sg, int m,
+                                             int M, int K, int Kpad, __half *__restrict__ dig, int *__restrict__ E, int *sparse) {
+    const int lane = threadIdx.x & 31;
     double x[NI][2];
-    unsigned int e = 0;
+    int ex[NI][2], em = 2 * OZ_SKIP;
+    bool bad = false, hole = false;
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
         const int k = 2 * (lane + 32 * i);
@@ -190,36 +213,60 @@ __global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, 
         x[i][1] = k + 1 < K ? row[(long long)(k + 1) * ks] : 0.0;
     }
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
-        e = max(e, max((unsigned int)__double2hiint(x[i][0]) & 0x7FF00000u, (unsigned int)__double2hiint(x[i][1]) & 0x7FF00000u));
-    const int em = max((int)(__reduce_max_sync(0xffffffffu, e) >> 20), 1);
-    if (lane == 0) E[m] = em;
+    for (int i = 0; i < NI; ++i) {
+        const int k = 2 * (lane + 32 * i);
+        const int2 s = k < Kpad ? *reinterpret_cast<const int2 *>(sh + k) : make_int2(OZ_SKIP, OZ_SKIP);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int sj = j ? s.y : s.x;
+            bad |= (__double2hiint(x[i][j]) & 0x7FF00000) == 0x7FF00000;
+            if (sj == OZ_SKIP) x[i][j] = 0.0;
+            hole |= sj != OZ_SKIP && x[i][j] == 0.0;
+            ex[i][j] = oz_exp((unsigned long long)__double_as_longlong(x[i][j]), sg * sj);
+            em = max(em, ex[i][j]);
+        }
+    }
+    em = __reduce_max_sync(0xffffffffu, em);
+    bad = __any_sync(0xffffffffu, bad);
+    hole = __any_sync(0xffffffffu, hole);
+    if (lane == 0) {
+        E[m] = bad ? OZ_NONFINITE : max(em, OZ_SKIP);
+        if (sparse && hole && em > OZ_SKIP) *sparse = 1;
+    }
     const long long DS = (long long)M * Kpad / 2;     // words per digit plane
     uint32_t *dst = reinterpret_cast<uint32_t *>(dig) + (long long)m * (Kpad / 2) + lane;
     const __half2 bias = __half2half2(__ushort_as_half(0x6480));   // 1152
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
         if (2 * (lane + 32 * i) >= Kpad) break;
-        const unsigned long long ua = oz_fixed((unsigned long long)__double_as_longlong(x[i][0]), em);
-        const unsigned long long ub = oz_fixed((unsigned long long)__double_as_longlong(x[i][1]), em);
+        const unsigned long long ua = oz_fixed((unsigned long long)__double_as_longlong(x[i][0]), em - ex[i][0]);
+        const unsigned long long ub = oz_fixed((unsigned long long)__double_as_longlong(x[i][1]), em - ex[i][1]);
         const uint32_t al = (uint32_t)ua, ah = (uint32_t)(ua >> 32), bl = (uint32_t)ub, bh = (uint32_t)(ub >> 32);
-        auto put = [&](int d, uint32_t v) {   // v: two FP16 words 1024 + digit + 128
+#pragma unroll
+        for (int d = 0; d < OZ_S; ++d) {   // two FP16 words 1024 + digit + 128, less 1152
+            const uint32_t v = (__byte_perm(d < 4 ? ah : al, d < 4 ? bh : bl, 0x0703 - 0x0101 * (d & 3)) & 0x00FF00FFu) | 0x64006400u;
             const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), bias);
             dst[d * DS + 32 * i] = *reinterpret_cast<const uint32_t *>(&h);
-        };
-        put(0, __byte_perm(ah, bh, 0x7632) + 0x64006400u);
-        put(1, (__byte_perm(ah, bh, 0x0501) & 0x00FF00FFu) | 0x64006400u);
-        put(2, (__byte_perm(ah, bh, 0x0400) & 0x00FF00FFu) | 0x64006400u);
-        put(3, (__byte_perm(al, bl, 0x0703) & 0x00FF00FFu) | 0x64006400u);
-        put(4, (__byte_perm(al, bl, 0x0602) & 0x00FF00FFu) | 0x64006400u);
-        put(5, (__byte_perm(al, bl, 0x0501) & 0x00FF00FFu) | 0x64006400u);
-        put(6, (__byte_perm(al, bl, 0x0400) & 0x00FF00FFu) | 0x64006400u);
+        }
     }
 }
 
-// launch of k_oz_split for M rows of K <= OZ_MAXK values: row pitch rs, value pitch ks (1, n for the rows and
-// columns of an n x n matrix); pdl: as a programmatic dependent launch
-inline void oz_split(const double *A, long long rs, int ks, int M, int K, __half *dig, int *E, int R, const int *active, int amod,
+// Bound by its 8 bytes read and 16 written per value, most of them in L2; a pass of its own because inside the
+// GEMM every column tile would split the rows again (measured there: 7,000 issue slots per 128 x 32 stage
+// against 3,100 cycles of MMAs).
+template <int NI>
+__global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, int M, int K, int Kpad, const int *__restrict__ sh,
+                                                  __half *__restrict__ dig, int *__restrict__ E, int R,
+                                                  const int *__restrict__ active, int amod) {
+    const int m = blockIdx.x * 8 + (threadIdx.x >> 5);
+    tc_pdl_enter();
+    if (m >= M) return;
+    if (active && !active[(m / R) % amod]) return;   // a frozen run's rows: their products are not used
+    oz_split_row<NI>(A + (long long)m * K, 1, sh, 1, m, M, K, Kpad, dig, E, nullptr);
+}
+
+// launch of k_oz_split for the M rows of A (K <= OZ_MAXK values each); pdl: as a programmatic dependent launch
+inline void oz_split(const double *A, int M, int K, const int *sh, __half *dig, int *E, int R, const int *active, int amod,
                      cudaStream_t st, bool pdl = false) {
     const int Kpad = oz_kpad(K);
     cudaLaunchConfig_t cfg = {};
@@ -231,8 +278,8 @@ inline void oz_split(const double *A, long long rs, int ks, int M, int K, __half
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
-    auto go = [&](void (*k)(const double *, long long, int, int, int, int, __half *, int *, int, const int *, int)) {
-        cudaLaunchKernelEx(&cfg, k, A, rs, ks, M, K, Kpad, dig, E, R, active, amod);   // errors: the caller's cudaGetLastError
+    auto go = [&](void (*k)(const double *, int, int, int, const int *, __half *, int *, int, const int *, int)) {
+        cudaLaunchKernelEx(&cfg, k, A, M, K, Kpad, sh, dig, E, R, active, amod);   // errors: the caller's cudaGetLastError
     };
     switch ((Kpad + 63) / 64) {
         case 1: go(k_oz_split<1>); break;
@@ -242,6 +289,53 @@ inline void oz_split(const double *A, long long rs, int ks, int M, int K, __half
         case 5: go(k_oz_split<5>); break;
         case 6: go(k_oz_split<6>); break;
         default: go(k_oz_split<8>);
+    }
+}
+
+// ---- digits of a caller's bases (the allocation-free solve), all four in two launches -------------------
+struct OzBases {
+    const double *B[4];      // n x n, row-major
+    int n[4];
+    int *sh[4];              // shifts of the rows, oz_kpad(n) entries
+    __half *dig[4];
+    int *F[4];
+    int *sparse;             // 1: a basis has zeros inside rows and columns that are not zero
+};
+
+// shifts: one warp per row of a basis.  Infinities and NaN (whose columns' results are NaN) set none.
+static __global__ void __launch_bounds__(256) k_oz_rows(OzBases g) {
+    const int b = blockIdx.y, k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, n = g.n[b];
+    if (blockIdx.x == 0 && b == 0 && threadIdx.x == 0) *g.sparse = 0;
+    if (k >= oz_kpad(n)) return;
+    int e = OZ_SKIP;
+    if (k < n)
+        for (int j = lane; j < n; j += 32) {
+            const unsigned long long u = (unsigned long long)__double_as_longlong(g.B[b][(long long)k * n + j]);
+            if (((u >> 52) & 0x7FF) != 0x7FF) e = max(e, oz_exp(u, -1023));
+        }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) g.sh[b][k] = e;
+}
+
+// digits: one warp per column, blockIdx.y the basis
+template <int NI>
+static __global__ void __launch_bounds__(256) k_oz_split_bases(OzBases g) {
+    const int b = blockIdx.y, m = blockIdx.x * 8 + (threadIdx.x >> 5), n = g.n[b];
+    if (m >= n) return;
+    oz_split_row<NI>(g.B[b] + m, n, g.sh[b], -1, m, n, n, oz_kpad(n), g.dig[b], g.F[b], g.sparse);
+}
+
+inline void oz_split_bases(const OzBases &g, cudaStream_t st) {   // errors: the caller's cudaGetLastError
+    int n = 0;
+    for (int v : g.n) n = v > n ? v : n;
+    k_oz_rows<<<dim3((unsigned)((oz_kpad(n) + 7) / 8), 4), 256, 0, st>>>(g);
+    const dim3 grid((unsigned)((n + 7) / 8), 4);
+    switch ((oz_kpad(n) + 63) / 64) {
+        case 1: k_oz_split_bases<1><<<grid, 256, 0, st>>>(g); break;
+        case 2: k_oz_split_bases<2><<<grid, 256, 0, st>>>(g); break;
+        case 3: k_oz_split_bases<3><<<grid, 256, 0, st>>>(g); break;
+        case 4: k_oz_split_bases<4><<<grid, 256, 0, st>>>(g); break;
+        default: k_oz_split_bases<8><<<grid, 256, 0, st>>>(g);
     }
 }
 
@@ -267,10 +361,10 @@ __device__ __forceinline__ bool oz_frozen(const OzArgs &g, int mt) {
 }
 
 // ---- the GEMM: persistent, warp-specialised; a CTA walks units of 128 rows x BN columns -------------
-//   warp 16     TMA: per 32-wide K stage the digits of A (32 x 128 x 7) and of B (32 x BN x 7), one 3D box each
-//   warps 17-18 issue the MMAs level by level (6 first), each level into a tensor-memory region of its own
-//               that it accumulates over a group of four stages: levels 6, 3, 2 by one warp, 5, 4, 1, 0 by
-//               the other, 28 MMAs of a stage each.  The drain of a level overlaps the group's later
+//   warp 16     TMA: per 32-wide K stage the digits of A (32 x 128 x 8) and of B (32 x BN x 8), one 3D box each
+//   warps 17-18 issue the MMAs level by level (7 first), each level into a tensor-memory region of its own
+//               that it accumulates over a group of four stages: levels 7, 6, 2 by one warp, 5, 4, 3, 1, 0 by
+//               the other, 36 MMAs of a stage each.  The drain of a level overlaps the group's later
 //               levels and the next group's first stage
 //   warps 0-15  drain the regions into the 64-bit integers, then convert and store (the epilogues of
 //               k_gemm).  Sixteen, because this code overflows the schedulers' instruction caches and its
@@ -280,6 +374,7 @@ __device__ __forceinline__ bool oz_frozen(const OzArgs &g, int mt) {
 // is freed and the kernel returns.
 static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_constant__ CUtensorMap tmA,
                                                                   const __grid_constant__ CUtensorMap tmB, OzArgs g) {
+    if (g.skip_if && *g.skip_if) return;
     extern __shared__ __align__(1024) unsigned char oz_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
     const int S = g.stages, BN = g.BN;
@@ -287,8 +382,8 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
     const uint32_t STAGE = OZ_ABYTES + OZ_S * BSL;
     double *outb = (double *)(base + (size_t)S * STAGE);
     uint64_t *bars = (uint64_t *)((unsigned char *)outb + OZ_OUTBYTES);
-    // barriers: full[4] (a stage's digits landed), empty[4] (both issuers' MMAs done with it), rfull[7] /
-    // rempty[7] (a level's group done / drained), fin[2]
+    // barriers: full[4] (a stage's digits landed), empty[4] (both issuers' MMAs done with it), rfull[8] /
+    // rempty[8] (a level's group done / drained), fin[2]
     const uint32_t b_full = smem_u32(bars), b_empty = b_full + 32, b_rfull = b_empty + 32, b_rempty = b_rfull + 8 * OZ_S,
                    b_fin = b_rempty + 8 * OZ_S;
     uint32_t *tslot = (uint32_t *)(bars + 8 + 2 * OZ_S + 2);
@@ -372,7 +467,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                     const bool first = (c & (OZ_GRP - 1)) == 0, last = (c & (OZ_GRP - 1)) == OZ_GRP - 1 || c == nst - 1;
 #pragma unroll
                     for (int d = OZ_S - 1; d >= 0; --d) {
-                        const bool mine = (d == 6 || d == 3 || d == 2) ? w == 0 : w == 1;
+                        const bool mine = (d == 7 || d == 6 || d == 2) ? w == 0 : w == 1;
                         if (!mine) continue;
                         if (first) {
                             if (!mbar_wait_warp(b_rempty + 8 * d, gph, abort_flag, g.wait_ns)) { fail(); ok = false; break; }
@@ -405,10 +500,11 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
             __syncwarp();
         }
     } else {
-        // ---- drain, epilogue (warps 0-7) ------------------------------------------------------------------
+        // ---- drain, epilogue (warps 0-15) ------------------------------------------------------------------
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REG_EPI));
         const int quarter = warp & 3, half = warp >> 2;   // 32 rows; which quarter of the columns
         long long acc[OZ_MAXH];
+        uint32_t frac[OZ_MAXH / 4] = {};   // a byte per column
 #pragma unroll
         for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
         uint32_t gph = 0;
@@ -419,8 +515,33 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
             const int hbn = (nt == ntn - 1 ? g.BNlast : BN) >> 2;   // columns per thread (8 or 16)
             const uint32_t lane0 = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * hbn);
             for (int c = 0; c < nst && ok; c += OZ_GRP, gph ^= 1u) {
+                // levels 7 and 6 together: what they add to acc, and a byte of fraction that stays
+                ok = mbar_wait(b_rfull + 8 * 7, gph, abort_flag, g.wait_ns) && mbar_wait(b_rfull + 8 * 6, gph, abort_flag, g.wait_ns);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                for (int d = OZ_S - 1; d >= 0; --d) {
+                for (int j0 = 0; j0 < OZ_MAXH; j0 += 8)
+                    if (j0 < hbn) {
+                        float lo[8], hi[8];
+                        tmem_ld8(lane0 + (uint32_t)(7 * BN + j0), lo);
+                        tmem_ld8(lane0 + (uint32_t)(6 * BN + j0), hi);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            uint32_t &f = frac[(j0 + j) >> 2];
+                            const int sh = 8 * (j & 3), t = __float2int_rn(hi[j]) + ((__float2int_rn(lo[j]) + 128) >> 8) + (int)((f >> sh) & 0xFF);
+                            acc[j0 + j] += t >> 8;
+                            f = (f & ~(0xFFu << sh)) | ((uint32_t)(t & 0xFF) << sh);
+                        }
+                    }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(b_rempty + 8 * 7);
+                    mbar_arrive(b_rempty + 8 * 6);
+                }
+#pragma unroll
+                for (int d = 5; d >= 0; --d) {
                     if (!mbar_wait(b_rfull + 8 * d, gph, abort_flag, g.wait_ns)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t ta = lane0 + (uint32_t)(d * BN);
@@ -435,11 +556,8 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                     for (int j0 = 0; j0 < OZ_MAXH; j0 += 8)
                         if (j0 < hbn) {
 #pragma unroll
-                            for (int j = j0; j < j0 + 8; ++j) {
-                                const int w = __float2int_rn(v[j]);   // an integer
-                                if (d == 6) acc[j] += (long long)((w + 128) >> 8);
-                                else acc[j] += (long long)w * (1ll << (8 * (5 - d)));
-                            }
+                            for (int j = j0; j < j0 + 8; ++j)   // integers
+                                acc[j] += (long long)__float2int_rn(v[j]) * (1ll << (8 * (5 - d)));
                         }
                 }
             }
@@ -456,7 +574,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
             const int fl = lane < ncol ? g.F[nb + lane] : 1;   // the exponents of the warp's columns, one per lane
             double *ob = outb + warp * (32 * OZ_OUTP);
             double *cb = g.C + ((long long)p * g.N + nb) * g.ldr + rr;   // store 1
-            const bool nan = em == 0x7FF || !ok;
+            const bool nan = em == OZ_NONFINITE || !ok;
             // store 0: this lane's place in a round's block, rows 8 i + lane / 4, column lane % 4
             const int lr = lane >> 2, lc = lane & 3;
             const double *rp[4] = {nullptr, nullptr, nullptr, nullptr};   // the reciprocals' rows
@@ -482,10 +600,10 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                         if (rp[i] && j0 + OZ_OUTC + lc < ncol) rn[i] = rp[i][j0 + OZ_OUTC];
                 }
 #pragma unroll
-                for (int j = 0; j < OZ_OUTC; ++j) {   // units 2^56 of X Y 2^(E + F - 2154)
+                for (int j = 0; j < OZ_OUTC; ++j) {   // units 2^64 of X Y 2^(E + F - 2168)
                     const int fn = __shfl_sync(0xffffffffu, fl, j0 + j);
-                    v[j] = oz_double(acc[j], em + fn - 2154 + 56);
-                    if (nan || fn == 0x7FF) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+                    v[j] = oz_double(acc[j], (int)((frac[0] >> (8 * j)) & 0xFF), em + fn - 2168 + 64);
+                    if (nan || fn == OZ_NONFINITE) v[j] = __longlong_as_double(0x7FF8000000000000ll);
                 }
                 if (g.store == 1) {             // lanes hold consecutive rows: coalesced as it is
 #pragma unroll
@@ -535,9 +653,13 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
                 }
 #pragma unroll
                 for (int j = 0; j + OZ_OUTC < OZ_MAXH; ++j) acc[j] = acc[j + OZ_OUTC];
+#pragma unroll
+                for (int j = 0; j + 1 < OZ_MAXH / 4; ++j) frac[j] = frac[j + 1];
             }
 #pragma unroll
             for (int j = 0; j < OZ_MAXH; ++j) acc[j] = 0;
+#pragma unroll
+            for (int j = 0; j < OZ_MAXH / 4; ++j) frac[j] = 0;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

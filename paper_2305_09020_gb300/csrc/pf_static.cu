@@ -25,12 +25,12 @@ namespace {
 static __device__ __align__(256) double g_fdm_scratch[2 * PF_STATIC_MAX_VALUES];
 
 // Digits of the right-hand sides and of the four eigenbases for the tensor-core transforms
-// (pf_oz.cuh), 43 MB in all: planes whose padded rows fit take those, others the FMA kernel.
+// (pf_oz.cuh), 49 MB in all: planes whose padded rows fit take those, others the FMA kernel.
 constexpr size_t DIG_A = (size_t)pf::OZ_S << 21, DIG_B = (size_t)pf::OZ_S * pf::OZ_MAXK * pf::OZ_MAXK;
 constexpr int DIG_ROWS = 1 << 16, DIG_MIN = 16;   // n_x, n_y >= 16: at most 2^16 rows of 2^20 values
 struct Digits {
     __half a[DIG_A], b[4][DIG_B];
-    int E[DIG_ROWS], F[4][pf::OZ_MAXK];
+    int E[DIG_ROWS], F[4][pf::OZ_MAXK], sh[4][pf::OZ_MAXK], sparse;
 };
 static __device__ __align__(256) unsigned char g_fdm_digits[sizeof(Digits)];
 
@@ -82,8 +82,10 @@ int scratch_for_current_device(double **out, Digits **digits, int *sms) {
 }
 
 int launch_gemm(const double *A, const double *B, double *C, long long rows, int n, int R, int store,
-                const double *lamN, const double *lamR, const double *cpl, int cpl_mod, cudaStream_t st) {
+                const double *lamN, const double *lamR, const double *cpl, int cpl_mod, cudaStream_t st,
+                const int *only_if = nullptr) {
     pf::GemmArgs<double> g{A, B, C, rows, n, R, store, lamN, lamR, cpl, cpl_mod};
+    g.only_if = only_if;
     dim3 grid((n + 63) / 64, (unsigned)((rows + 63) / 64));
     pf::k_gemm<double, 64, 64, 8, 4, 4><<<grid, 256, 0, st>>>(g);
     cudaError_t e = cudaGetLastError();
@@ -99,7 +101,7 @@ int launch_digits(Digits *D, int sms, const double *A, int b, double *C, long lo
                   const double *lamN, const double *lamR, const double *cpl, int cpl_mod, cudaStream_t st) {
     size_t smem = 0;
     pf::OzArgs a = pf::oz_plan(rows, n, sms, &smem);
-    a.E = D->E; a.F = D->F[b];
+    a.E = D->E; a.F = D->F[b]; a.skip_if = &D->sparse;
     a.R = R; a.store = store; a.ldc = n; a.ldr = R;
     a.lamN = lamN; a.lamR = lamR; a.cpl = cpl; a.cpl_mod = cpl_mod;
     a.C = C;
@@ -109,7 +111,7 @@ int launch_digits(Digits *D, int sms, const double *A, int b, double *C, long lo
         pf_internal_set_error("cuTensorMapEncodeTiled failed");
         return PF_ECUDA;
     }
-    pf::oz_split(A, n, 1, (int)rows, n, D->a, D->E, R, nullptr, 1, st);
+    pf::oz_split(A, (int)rows, n, D->sh[b], D->a, D->E, R, nullptr, 1, st);
     pf::k_gemm_oz<<<(unsigned)(a.nunits < sms ? a.nunits : sms), pf::OZ_THREADS, smem, st>>>(ma, mb, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -119,8 +121,9 @@ int launch_digits(Digits *D, int sms, const double *A, int b, double *C, long lo
     return PF_OK;
 }
 
-// The tensor-core transforms take twelve launches (the eigenbases are split anew in each call: they
-// are the caller's) against four, and are the faster ones from the smallest planes measured on: 32 x 17 nodes,
+// The tensor-core transforms take ten launches (the eigenbases are split anew in each call: they
+// are the caller's) and the four of the FMA kernels, which return at once unless a basis falls into uncoupled
+// pieces, and are the faster ones from the smallest planes measured on: 32 x 17 nodes,
 // one plane 149 -> 80 us; 128 x 65, one plane 451 -> 107 us, 64 planes 607 -> 133 us; 240 x 121, 30 planes
 // 1547 -> 170 us.
 bool digits_fit(int nx, int ny, long long total) {
@@ -153,20 +156,21 @@ extern "C" int pf_fdm_solve_static(int nx, int ny, int nplanes, const double *Sx
     double *W1 = scratch, *W2 = scratch + PF_STATIC_MAX_VALUES;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const long long P = nplanes;
+    const int *fma = nullptr;
     if (digits_fit(nx, ny, total)) {
-        // digits of each eigenbasis by columns
-        pf::oz_split(Sx, 1, nx, nx, nx, D->b[0], D->F[0], 1, nullptr, 1, st);
-        pf::oz_split(Sy, 1, ny, ny, ny, D->b[1], D->F[1], 1, nullptr, 1, st);
-        pf::oz_split(SyT, 1, ny, ny, ny, D->b[2], D->F[2], 1, nullptr, 1, st);
-        pf::oz_split(SxT, 1, nx, nx, nx, D->b[3], D->F[3], 1, nullptr, 1, st);
+        // shifts and digits of each eigenbasis by columns
+        pf::OzBases g{{Sx, Sy, SyT, SxT}, {nx, ny, ny, nx}, {}, {}, {}, &D->sparse};
+        for (int b = 0; b < 4; ++b) g.sh[b] = D->sh[b], g.dig[b] = D->b[b], g.F[b] = D->F[b];
+        pf::oz_split_bases(g, st);
         if ((rc = launch_digits(D, sms, rhs, 0, W1, P * ny, nx, ny, 1, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
         if ((rc = launch_digits(D, sms, W1, 1, W2, P * nx, ny, nx, 0, lam_y, lam_x, shift, nplanes, st)) != PF_OK) return rc;
         if ((rc = launch_digits(D, sms, W2, 2, W1, P * nx, ny, nx, 1, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
-        return launch_digits(D, sms, W1, 3, out, P * ny, nx, ny, 0, nullptr, nullptr, nullptr, 1, st);
+        if ((rc = launch_digits(D, sms, W1, 3, out, P * ny, nx, ny, 0, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
+        fma = &D->sparse;   // the kernels below run only where a basis falls into uncoupled pieces
     }
     // the same four transforms as the handle's solves: x, y (+ eigenvalue division), y^T, x^T
-    if ((rc = launch_gemm(rhs, Sx, W1, P * ny, nx, ny, 1, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
-    if ((rc = launch_gemm(W1, Sy, W2, P * nx, ny, nx, 0, lam_y, lam_x, shift, nplanes, st)) != PF_OK) return rc;
-    if ((rc = launch_gemm(W2, SyT, W1, P * nx, ny, nx, 1, nullptr, nullptr, nullptr, 1, st)) != PF_OK) return rc;
-    return launch_gemm(W1, SxT, out, P * ny, nx, ny, 0, nullptr, nullptr, nullptr, 1, st);
+    if ((rc = launch_gemm(rhs, Sx, W1, P * ny, nx, ny, 1, nullptr, nullptr, nullptr, 1, st, fma)) != PF_OK) return rc;
+    if ((rc = launch_gemm(W1, Sy, W2, P * nx, ny, nx, 0, lam_y, lam_x, shift, nplanes, st, fma)) != PF_OK) return rc;
+    if ((rc = launch_gemm(W2, SyT, W1, P * nx, ny, nx, 1, nullptr, nullptr, nullptr, 1, st, fma)) != PF_OK) return rc;
+    return launch_gemm(W1, SxT, out, P * ny, nx, ny, 0, nullptr, nullptr, nullptr, 1, st, fma);
 }
