@@ -276,7 +276,7 @@ struct Engine {
     struct OzRcp {
         int bcset;
         const T *sh;
-        double *rcp;
+        double2 *rcp;
     };
     std::vector<OzRcp> ozrcp;
     __half *ozdig = nullptr;
@@ -616,8 +616,8 @@ struct Engine {
         ozb.push_back(t);
     }
     void add_rcp(int bcset, const T *sh) {
-        const int modes = d3 ? nz / 2 + 1 : 1;
-        double *q = mk<double>((size_t)modes * nx * ny);
+        const int modes = d3 ? nz / 2 + 1 : 1;   // modes nx ny < 2^31: at most 513 planes of 480^2
+        double2 *q = mk<double2>((size_t)modes * nx * ny);
         pf::k_oz_rcp<<<1024, 256, 0, st>>>(q, reinterpret_cast<const double *>(Ly[bcset]), reinterpret_cast<const double *>(Lx),
                                            reinterpret_cast<const double *>(sh), modes, nz, nx, ny);
         check_launch();
@@ -634,7 +634,7 @@ struct Engine {
         return m.map;
     }
     void gemm_oz(const T *A, const T *B, T *C, long long rows, int R, int store, const T *lamN, const T *lamR,
-                 const T *cpl, const double *rcp, T *C2 = nullptr, const T *face2 = nullptr) {
+                 const T *cpl, const double2 *rcp, T *C2 = nullptr, const T *face2 = nullptr) {
         const OzB *ob = nullptr;
         for (auto &t : ozb)
             if (t.key == B) ob = &t;
@@ -666,7 +666,7 @@ struct Engine {
         prof->end(st);
     }
     void fdm_oz(const T *rhs, T *out, int bcset, const T *sh, long long P, T *minus_m_out, const T *face) {
-        const double *rcp = nullptr;
+        const double2 *rcp = nullptr;
         for (auto &r : ozrcp)
             if (r.bcset == bcset && r.sh == sh) rcp = r.rcp;
         gemm_oz(rhs, Sx, W1, P * ny, ny, 1, nullptr, nullptr, nullptr, nullptr);

@@ -77,8 +77,8 @@ struct OzArgs {
     int R, store, ldc, ldr;
     const double *lamN, *lamR, *cpl;   // optional division by lamN[n] + lamR[r] + cpl[p % cpl_mod]
     int cpl_mod;
-    const double *rcp;        // its reciprocals [mode][r][n], mode of plane p: 0 when rcp_modes == 1, else
-    int rcp_modes;            // that of the packed Fourier plane p % cpl_mod; null: divide
+    const double2 *rcp;       // its reciprocals (oz_recip) [mode][r][n], mode of plane p: 0 when rcp_modes == 1,
+    int rcp_modes;            // else that of the packed Fourier plane p % cpl_mod; null: divide
     double *C;
     double *C2;               // optional C2[m ldc + n] = -m2x[n] m2y[r] C (+ face2[p N + n] on r == 0)
     const double *m2x, *m2y, *face2;
@@ -193,6 +193,16 @@ __device__ __forceinline__ double oz_double(long long acc, int frac, int sc) {
     }
     return __hiloint2double(hi + (int)((unsigned)sc << 20), __double2loint(x));
 }
+
+// 1/d as a rounded reciprocal and what it leaves (0 for d = 0, whose quotients are 0), and x/d from them: the
+// product with both is x/d to 2^-100 before it is rounded, once, as the division operator rounds.  The
+// rounded reciprocal alone leaves up to 1.5 units in the last place.
+__host__ __device__ __forceinline__ double2 oz_recip(double d) {
+    if (d == 0.0) return double2{0.0, 0.0};
+    const double r = 1.0 / d, lo = fma(-r, d, 1.0) * r;
+    return double2{r, lo == lo ? lo : 0.0};
+}
+__host__ __device__ __forceinline__ double oz_quot(double x, double2 r) { return fma(x, r.x, x * r.y); }
 
 #ifndef PF_OZ_HELPERS_ONLY
 // ---- digits of A: one warp per row ----------------------------------------------------------------
@@ -339,16 +349,15 @@ inline void oz_split_bases(const OzBases &g, cudaStream_t st) {   // errors: the
     }
 }
 
-// reciprocals of the eigenvalue sums of one solve family, [mode][r][n] (0 where a sum is 0)
-static __global__ void k_oz_rcp(double *__restrict__ out, const double *__restrict__ lamN, const double *__restrict__ lamR,
+// reciprocals of the eigenvalue sums of one solve family, [mode][r][n]
+static __global__ void k_oz_rcp(double2 *__restrict__ out, const double *__restrict__ lamN, const double *__restrict__ lamR,
                                 const double *__restrict__ shift, int modes, int nz, int R, int N) {
     const long long n = (long long)modes * R * N;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const int k = (int)(i / ((long long)R * N));
         const int r = (int)(i / N - (long long)k * R), c = (int)(i % N);
         const int p = modes == 1 ? 0 : k == 0 ? 0 : (k == nz / 2 ? 1 : 2 * k);   // a packed plane of mode k
-        const double d = lamN[c] + lamR[r] + shift[p];
-        out[i] = d != 0.0 ? 1.0 / d : 0.0;
+        out[i] = oz_recip(lamN[c] + lamR[r] + shift[p]);
     }
 }
 
@@ -577,27 +586,24 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
             const bool nan = em == OZ_NONFINITE || !ok;
             // store 0: this lane's place in a round's block, rows 8 i + lane / 4, column lane % 4
             const int lr = lane >> 2, lc = lane & 3;
-            const double *rp[4] = {nullptr, nullptr, nullptr, nullptr};   // the reciprocals' rows
-            double rc[4] = {1.0, 1.0, 1.0, 1.0};
+            int ro[4] = {-1, -1, -1, -1};   // the reciprocals of those rows at column lc (-1: none)
             if (g.rcp) {
                 const int pl = p % g.cpl_mod, md = g.rcp_modes == 1 ? 0 : (pl == 1 ? g.cpl_mod / 2 : pl >> 1);
-                const int q = m < g.M ? md * g.R + rr : -1;
+                const int q = m < g.M ? (md * g.R + rr) * g.N + nb : -1;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int row = __shfl_sync(0xffffffffu, q, 8 * i + lr);
-                    if (row >= 0) {
-                        rp[i] = g.rcp + (long long)row * g.N + nb + lc;
-                        if (lc < ncol) rc[i] = *rp[i];
-                    }
+                    ro[i] = __shfl_sync(0xffffffffu, q, 8 * i + lr);
+                    if (ro[i] >= 0) ro[i] += lc;
                 }
             }
 #pragma unroll 1
             for (int j0 = 0; j0 < ncol; j0 += OZ_OUTC) {
-                double v[OZ_OUTC], rn[4] = {1.0, 1.0, 1.0, 1.0};
-                if (g.rcp) {   // the next round's reciprocals in flight during this one
+                double v[OZ_OUTC];
+                double2 rc[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (rp[i] && j0 + OZ_OUTC + lc < ncol) rn[i] = rp[i][j0 + OZ_OUTC];
+                for (int i = 0; i < 4; ++i) {   // in flight during the conversions
+                    rc[i] = double2{1.0, 0.0};
+                    if (ro[i] >= 0 && j0 + lc < ncol) rc[i] = g.rcp[ro[i] + j0];
                 }
 #pragma unroll
                 for (int j = 0; j < OZ_OUTC; ++j) {   // units 2^64 of X Y 2^(E + F - 2168)
@@ -621,8 +627,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         v[i] = ob[(8 * i + lr) * OZ_OUTP + lc];
-                        if (g.rcp) v[i] *= rc[i];
-                        rc[i] = rn[i];
+                        if (g.rcp) v[i] = oz_quot(v[i], rc[i]);
                     }
                     if (plain) {
 #pragma unroll
