@@ -165,7 +165,7 @@ int pf_fdm_1d(int n, const double *Kmat, const double *Mdiag, const unsigned cha
  * cuda_stream: a cudaStream_t (NULL = legacy default stream).
  * Errors: PF_EINVAL (bad descriptor, including patch intervals that are not finite with
  * x0 <= x1, PF_BC_PATCHES on the top, or a potential with no Dirichlet node at all),
- * PF_ENOMEM, PF_ECUDA. *out is NULL on error. */
+ * PF_ENOMEM, PF_ECUDA, PF_ETIMEOUT (a bounded device-side wait gave up). *out is NULL on error. */
 int pf_create(const pf_mesh *mesh, const pf_fluid *fluid, const pf_vbc *vbc,
               const pf_scheme *scheme, const double *phi0, const double *u0,
               void *cuda_stream, pf_handle **out);
@@ -178,7 +178,8 @@ int pf_step(pf_handle *h, int nsteps);
 /* Synchronise the handle's stream and check the state for non-finite values:
  * returns PF_EDIVERGED if any was found since creation.  Returns PF_ETIMEOUT (and clears the
  * condition) when a bounded device-side wait of the tensor-core transforms gave up since the
- * last pf_sync; the fields computed by those steps are then not valid. */
+ * last pf_sync; the fields computed by those steps are then not valid.  pf_get_fields,
+ * pf_diagnostics and pf_autotune return PF_ETIMEOUT too while the condition stands, without clearing it. */
 int pf_sync(pf_handle *h);
 
 /* Copy fields to the host (synchronous).  mask: PF_FIELD_* bits; blocks of
@@ -316,8 +317,9 @@ int pf_set_tc_accum(pf_handle *h, int gemm, int family, int slices, int sep);
 /* Test hook of the failure detection (Sec. 3 has no counterpart): the next tensor-core transform
  * launch of h waits on a device barrier that nothing arrives at, gives up after wait_ns
  * nanoseconds (0 < wait_ns <= 1e10), records the time-out in the handle's error word and returns
- * without touching tensor memory; pf_sync (after pf_step) or pf_solve_helmholtz then return
- * PF_ETIMEOUT.  The next pf_step runs without its captured graph so that the hook applies.
+ * without touching tensor memory; pf_sync, pf_get_fields or pf_diagnostics (after pf_step) or
+ * pf_solve_helmholtz then return PF_ETIMEOUT.  The next pf_step runs without its captured graph so that
+ * the hook applies.
  * PF_EINVAL when the handle does not use the tensor-core transforms. */
 int pf_debug_tc_stall(pf_handle *h, unsigned long long wait_ns);
 
@@ -337,7 +339,10 @@ typedef struct pf_batch pf_batch;
 /* meshes/fluids/vbcs: nrun descriptors each (nz must be 1); scheme shared by all runs;
  * phi0[r]: host array of run r's n_x*n_y initial phase field.  Each group computes its
  * initial potentials by the fixed point of the Remark in Sec. 3.1 (FP64).  Errors: PF_EINVAL
- * (message in pf_last_error(NULL)), PF_ENOMEM, PF_ECUDA. */
+ * (message in pf_last_error(NULL)), PF_ENOMEM, PF_ECUDA, PF_ETIMEOUT.
+ * When a bounded device-side wait of the tensor-core transforms gives up, the calls below that read results
+ * or wait for the GPU return PF_ETIMEOUT from then on, as does pf_batch_step once it is known: the state is not
+ * valid and cannot be written again. */
 int pf_batch_create(int nrun, const pf_mesh *meshes, const pf_fluid *fluids, const pf_vbc *vbcs,
                     const pf_scheme *scheme, const double *const *phi0, void *cuda_stream, pf_batch **out);
 
@@ -368,6 +373,10 @@ int pf_batch_autotune(pf_batch *b, int steps, double *ms_out);
 /* Pin the transform variant of every group (codes as pf_set_variant); PF_EINVAL, nothing
  * changed, when some group cannot use it. */
 int pf_batch_set_variant(pf_batch *b, int gemm, int fuse_y);
+
+/* Test hook as pf_debug_tc_stall, for the next tensor-core transform of one group (its next step runs
+ * without the captured graph).  PF_EINVAL when no group uses the tensor-core transforms. */
+int pf_batch_debug_tc_stall(pf_batch *b, unsigned long long wait_ns);
 
 /* Message of the ensemble's last failed call (empty if none; pf_last_error(NULL)'s message for
  * b == NULL).  The string is owned by the ensemble and valid until its next call. */

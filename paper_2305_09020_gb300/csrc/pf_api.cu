@@ -221,7 +221,9 @@ struct Engine {
     int *active = nullptr, *run_count = nullptr, *steps_at = nullptr;
     double *tol_dev = nullptr;
     double *red;
-    int *dev_err;   // device error word (bounded waits)
+    // error word of the bounded waits, in mapped host memory: the host reads it wherever it has waited for the
+    // stream anyway, without a copy
+    int *host_err = nullptr, *dev_err = nullptr;
     int cur = 0;
     // 3xTF32 tensor-core transforms: for each B matrix (an eigenbasis or its transpose), B^T split
     // into TF32 head and tail, zero padded to Npad x Kpad, with its TMA descriptors
@@ -519,7 +521,9 @@ struct Engine {
         }
 
         red = mk<double>(std::max<long long>(1024, nz));
-        dev_err = mk<int>(1);
+        PF_CU(cudaHostAlloc(&host_err, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable));
+        *host_err = 0;
+        PF_CU(cudaHostGetDevicePointer(&dev_err, host_err, 0));
         use_tc = (sizeof(T) == 4) && s.precision == PF_MIXED && tc_possible();
         if (use_tc) {
             // B = Sx (Bt = Sx^T), B = Sx^T (Bt = Sx), B = Sy (Bt = Sy^T), B = Sy^T (Bt = Sy)
@@ -653,7 +657,10 @@ struct Engine {
         a.m2x = reinterpret_cast<const double *>(Mx); a.m2y = reinterpret_cast<const double *>(My);
         a.face2 = reinterpret_cast<const double *>(face2);
         a.active = active; a.amod = nz;
-        a.err = dev_err; a.wait_ns = tc_wait_ns;
+        a.err = dev_err;
+        a.wait_ns = tc_stall ? tc_wait_ns_next : tc_wait_ns;
+        a.stall = tc_stall;
+        tc_stall = 0;
         const CUtensorMap ma = ozmap(ozdig, rows, ob->Kpad, pf::OZ_BM), mb = ozmap(ob->dig, N, ob->Kpad, a.BN);
         const double *A64 = reinterpret_cast<const double *>(A);
         prof->begin(PF_KC_GEMM, st);
@@ -819,6 +826,7 @@ struct Engine {
         for (int c = 0; c < 2; ++c)
             if (graph[c]) cudaGraphExecDestroy(graph[c]);
         for (void *q : allocs) cudaFree(q);
+        if (host_err) cudaFreeHost(host_err);
     }
 
     // ensembles: every run active, no exit recorded, step counts `count`, tolerance tol (< 0: only
@@ -1371,13 +1379,20 @@ struct Engine {
         return acc * (d3 ? hs.lz / nz : 1.0);
     }
 
-    // error word of the bounded device waits: read (synchronous) and clear
+    // error word of the bounded device waits: of the work that the stream has been waited for; with clearing
+    int peek_err() const { return *(volatile int *)host_err; }
     int take_err() {
-        int e = 0;
-        PF_CU(cudaMemcpyAsync(&e, dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
         PF_CU(cudaStreamSynchronize(st));
-        if (e) PF_CU(cudaMemsetAsync(dev_err, 0, sizeof(int), st));
+        const int e = peek_err();
+        if (e) *(volatile int *)host_err = 0;
         return e;
+    }
+    // the next tensor-core transform launch reports a time-out after wait_ns; false without such transforms
+    bool stall_next(unsigned long long wait_ns) {
+        if (!(use_tc && !tcb.empty()) && !use_oz) return false;
+        tc_stall = 1;
+        tc_wait_ns_next = wait_ns;
+        return true;
     }
 
     // ---- reductions (FP64 accumulation) -------------------------------------------------------
@@ -1429,6 +1444,8 @@ int fail(pf_handle *h, int code, const std::string &msg) {
 int cuda_fail(pf_handle *h, const CudaError &e) {
     return fail(h, PF_ECUDA, e.where + ": " + cudaGetErrorString(e.code));
 }
+
+const char *const TIMEOUT_MSG = "a tensor-core transform gave up waiting (bounded mbarrier wait)";
 
 void build_patches(HostSetup &s);
 
@@ -1609,6 +1626,10 @@ int initial_potential(const HostSetup &hs, Engine<double> &E, const double *phi0
         if (!(diff == diff)) {
             err = "non-finite value in the initial potential";
             return PF_EDIVERGED;
+        }
+        if (E.take_err()) {
+            err = TIMEOUT_MSG;
+            return PF_ETIMEOUT;
         }
         if (diff <= tol * vmax || (diff <= 1e-11 * vmax && diff >= prev)) break;
         prev = diff;
@@ -1847,8 +1868,7 @@ int sync_impl(pf_handle *h, Engine<T> &E) {
     for (int c = 0; c < 3; ++c)
         if (E.u[c][n]) um = std::max(um, E.reduce(E.u[c][n], nullptr, 1));
     if (E.take_err())
-        return fail(h, PF_ETIMEOUT, "a tensor-core transform gave up waiting (bounded mbarrier wait); the state "
-                                    "of the steps since the last pf_sync is not valid");
+        return fail(h, PF_ETIMEOUT, std::string(TIMEOUT_MSG) + "; the state of the steps since the last pf_sync is not valid");
     if (!(m == m) || !(um == um) || std::isinf(m) || std::isinf(um)) h->diverged = true;
     return h->diverged ? fail(h, PF_EDIVERGED, "non-finite value in the state") : PF_OK;
 }
@@ -1990,8 +2010,9 @@ int set_impl(pf_handle *h, Engine<T> &E, unsigned mask, const double *in, size_t
 extern "C" int pf_get_fields(pf_handle *h, unsigned mask, double *host_out, size_t n) {
     if (!h || !host_out) return PF_EINVAL;
     try {
-        if (h->e64) return get_impl(h, *h->e64, mask, host_out, n);
-        return get_impl(h, *h->e32, mask, host_out, n);
+        const int rc = h->e64 ? get_impl(h, *h->e64, mask, host_out, n) : get_impl(h, *h->e32, mask, host_out, n);
+        if (rc == PF_OK && (h->e64 ? h->e64->peek_err() : h->e32->peek_err())) return fail(h, PF_ETIMEOUT, TIMEOUT_MSG);
+        return rc;
     } catch (const CudaError &e) {
         return cuda_fail(h, e);
     }
@@ -2028,7 +2049,7 @@ int diag_impl(pf_handle *h, Engine<T> &E, double *out) {
     out[5] = h->diverged ? 1.0 : 0.0;
     out[6] = E.reduce(E.phi[n], E.phi[1 - n], 2) / h->hs.dt;
     out[7] = E.energy();
-    return PF_OK;
+    return E.peek_err() ? fail(h, PF_ETIMEOUT, TIMEOUT_MSG) : PF_OK;
 }
 
 template <typename T>
@@ -2052,7 +2073,7 @@ int helm_impl(pf_handle *h, Engine<T> &E, int bcset, int mode, double lambda, co
     PF_CU(cudaMemcpyAsync(o.data(), E.OUT, o.size() * sizeof(T), cudaMemcpyDeviceToHost, E.st));
     PF_CU(cudaStreamSynchronize(E.st));
     for (size_t i = 0; i < o.size(); ++i) out[i] = (double)o[i];
-    if (E.take_err()) return fail(h, PF_ETIMEOUT, "a tensor-core transform gave up waiting (bounded mbarrier wait)");
+    if (E.take_err()) return fail(h, PF_ETIMEOUT, TIMEOUT_MSG);
     return PF_OK;
 }
 }  // namespace
@@ -2197,6 +2218,8 @@ extern "C" int pf_autotune(pf_handle *h, int steps, int *choice, double *ms_per_
         h->nstep += total;
         h->t += total * h->hs.dt;
         h->last_J = 2;
+        PF_CU(cudaStreamSynchronize(h->st));
+        if (h->e64 ? h->e64->peek_err() : h->e32->peek_err()) return fail(h, PF_ETIMEOUT, TIMEOUT_MSG);
     } catch (const CudaError &e) {
         return cuda_fail(h, e);
     }
@@ -2263,11 +2286,9 @@ extern "C" int pf_set_step(pf_handle *h, int nstep, double t) {
 
 extern "C" int pf_debug_tc_stall(pf_handle *h, unsigned long long wait_ns) {
     if (!h) return PF_EINVAL;
-    if (!h->e32 || !h->e32->use_tc || h->e32->tcb.empty())
-        return fail(h, PF_EINVAL, "the handle does not run its transforms on the tensor cores");
     if (wait_ns == 0 || wait_ns > 10000000000ull) return fail(h, PF_EINVAL, "wait_ns must be in (0, 1e10]");
-    h->e32->tc_stall = 1;
-    h->e32->tc_wait_ns_next = wait_ns;
+    if (!(h->e64 ? h->e64->stall_next(wait_ns) : h->e32->stall_next(wait_ns)))
+        return fail(h, PF_EINVAL, "the handle does not run its transforms on the tensor cores");
     return PF_OK;
 }
 
@@ -2355,6 +2376,14 @@ int batch_fail(pf_batch *b, int code, const std::string &m) {
     return code;
 }
 
+// time-outs of the groups' bounded waits so far (of work that has been waited for, all of them).  The word stays
+// set: the state of an ensemble cannot be written again.
+int batch_timeout(pf_batch *b) {
+    for (auto &g : b->groups)
+        if (g->e64 ? g->e64->peek_err() : g->e32->peek_err()) return batch_fail(b, PF_ETIMEOUT, TIMEOUT_MSG);
+    return PF_OK;
+}
+
 void batch_invalidate_graphs(pf_batch *b) {
     for (int c = 0; c < 2; ++c)
         if (b->graph[c]) {
@@ -2377,7 +2406,9 @@ void batch_step_groups(pf_batch *b, int J) {
 
 void batch_step_once(pf_batch *b) {
     const int J = (b->nstep == 0 || b->bdf == 1) ? 1 : 2;
-    if (J == 1 || b->st == nullptr) {
+    bool stall = false;   // the test hook applies to kernels launched now
+    for (auto &g : b->groups) for_engine(*g, [&](auto &E) { stall = stall || E.tc_stall; });
+    if (J == 1 || b->st == nullptr || stall) {
         batch_step_groups(b, J);
     } else {
         int c = 0;
@@ -2490,6 +2521,7 @@ extern "C" int pf_batch_create(int nrun, const pf_mesh *meshes, const pf_fluid *
 
 extern "C" int pf_batch_step(pf_batch *b, int nsteps) {
     if (!b || nsteps < 0) return PF_EINVAL;
+    if (const int rc = batch_timeout(b)) return rc;
     try {
         for (int s = 0; s < nsteps; ++s) batch_step_once(b);
     } catch (const CudaError &e) {
@@ -2525,7 +2557,7 @@ extern "C" int pf_batch_umax(pf_batch *b, double *umax, double *mass) {
     } catch (const CudaError &e) {
         return batch_fail(b, PF_ECUDA, e.where + ": " + cudaGetErrorString(e.code));
     }
-    return PF_OK;
+    return batch_timeout(b);
 }
 
 extern "C" int pf_batch_run_to_equilibrium(pf_batch *b, double tol, int max_steps, int check_every, int *steps_out) {
@@ -2546,6 +2578,7 @@ extern "C" int pf_batch_run_to_equilibrium(pf_batch *b, double tol, int max_step
                     PF_CU(cudaStreamSynchronize(E.st));
                     for (int v : act) any = any || v;
                 });
+            if (const int rc2 = batch_timeout(b)) return rc2;
             if (!any) break;
         }
         for (auto &g : b->groups)
@@ -2608,7 +2641,7 @@ extern "C" int pf_batch_get_fields(pf_batch *b, int run, unsigned mask, double *
     } catch (const CudaError &e) {
         return batch_fail(b, PF_ECUDA, e.where + ": " + cudaGetErrorString(e.code));
     }
-    return PF_OK;
+    return batch_timeout(b);
 }
 
 extern "C" const char *pf_batch_last_error(const pf_batch *b) {
@@ -2682,10 +2715,20 @@ extern "C" int pf_batch_autotune(pf_batch *b, int steps, double *ms_out) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         batch_invalidate_graphs(b);
+        for (auto &g : b->groups) PF_CU(cudaStreamSynchronize(g->gst));
+        if (const int rc = batch_timeout(b)) return rc;
     } catch (const CudaError &e) {
         return batch_fail(b, PF_ECUDA, e.where + ": " + cudaGetErrorString(e.code));
     }
     return (int)b->groups.size();
+}
+
+extern "C" int pf_batch_debug_tc_stall(pf_batch *b, unsigned long long wait_ns) {
+    if (!b) return PF_EINVAL;
+    if (wait_ns == 0 || wait_ns > 10000000000ull) return batch_fail(b, PF_EINVAL, "wait_ns must be in (0, 1e10]");
+    for (auto &g : b->groups)   // one group is enough
+        if (g->e64 ? g->e64->stall_next(wait_ns) : g->e32->stall_next(wait_ns)) return PF_OK;
+    return batch_fail(b, PF_EINVAL, "no group runs its transforms on the tensor cores");
 }
 
 extern "C" int pf_batch_groups(const pf_batch *b, int *group_of) {

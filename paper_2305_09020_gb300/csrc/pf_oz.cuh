@@ -87,6 +87,7 @@ struct OzArgs {
     const int *skip_if;       // nullable: nothing is done where it holds a value that is not 0
     int *err;                 // error word; null: a call without one, whose results become NaN on a time-out
     unsigned long long wait_ns;
+    int stall;                // test hook: wait on a barrier that nothing arrives at, report, return
 };
 
 constexpr size_t OZ_SMEM = 227 * 1024;
@@ -413,6 +414,13 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (g.stall) {
+        __syncthreads();
+        tc_pdl_enter();
+        if (tid == 0 && !mbar_wait(b_fin, 0u, abort_flag, g.wait_ns)) tc_report(g.err);
+        __syncthreads();
+        return;
+    }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(g.tmem_cols)
@@ -425,7 +433,7 @@ static __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const __grid_c
     const uint32_t tmem = *tslot;
     tc_pdl_enter();   // everything above is this kernel's own
     auto fail = [&]() {
-        if (!*abort_flag && g.err) atomicExch(g.err, TC_ERR_TIMEOUT);
+        if (!*abort_flag && g.err) tc_report(g.err);
         *abort_flag = 1;
     };
     const int ntn = g.ntn, nst = g.nst;

@@ -178,6 +178,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, const 
     }
 }
 
+// a wait gave up: the error word lies in mapped host memory, and every writer writes the same value
+__device__ __forceinline__ void tc_report(int *err) { *(volatile int *)err = TC_ERR_TIMEOUT; }
+
 // The same wait by a whole warp, with one answer for all its lanes (elect.sync needs the warp whole)
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t mbar, uint32_t parity, const volatile int *abort,
                                                unsigned long long limit_ns) {
@@ -333,7 +336,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_pdl_enter();   // everything above is this kernel's own
     if (g.stall) {   // test hook: nothing arrives at b_stall; report the time-out and leave
         __syncthreads();
-        if (tid == 0 && !mbar_wait(b_stall, 0u, abort_flag, g.wait_ns)) atomicExch(g.err, TC_ERR_TIMEOUT);
+        if (tid == 0 && !mbar_wait(b_stall, 0u, abort_flag, g.wait_ns)) tc_report(g.err);
         return;
     }
     if (warp == 0) {
@@ -350,7 +353,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int my_tiles = g.ntiles > (int)blockIdx.x ? (g.ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int Q = my_tiles * nchunk;   // K chunks this CTA walks (stage of chunk q: q mod S)
     auto fail = [&]() {
-        if (!*abort_flag) atomicExch(g.err, TC_ERR_TIMEOUT);
+        if (!*abort_flag) tc_report(g.err);
         *abort_flag = 1;
     };
 

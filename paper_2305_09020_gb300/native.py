@@ -109,6 +109,7 @@ def load(build_if_missing: bool = True):
     L.pf_batch_set_variant.argtypes = [c_void_p, c_int, c_int]
     L.pf_batch_last_error.argtypes = [c_void_p]
     L.pf_batch_last_error.restype = c_char_p
+    L.pf_batch_debug_tc_stall.argtypes = [c_void_p, ctypes.c_ulonglong]
     L.pf_batch_groups.argtypes = [c_void_p, POINTER(c_int)]
     L.pf_batch_destroy.argtypes = [c_void_p]
     L.pf_batch_destroy.restype = None
@@ -422,6 +423,10 @@ class Batch:
         rc = load().pf_batch_set_variant(self._h, int(gemm), int(bool(fuse_y)))
         if rc < 0:
             _check_b(rc, self._h)
+
+    def debug_tc_stall(self, wait_ns: int):
+        """Test hook: the next tensor-core transform of one group reports a time-out after wait_ns."""
+        _check_b(load().pf_batch_debug_tc_stall(self._h, int(wait_ns)), self._h)
 
     def autotune(self, steps: int = 5):
         ng, _ = self.groups()
