@@ -164,8 +164,8 @@ class ClockSampler:
 def transform_kernel(code, fused_y):
     """Kernel(s) of the chosen transform variant (PF_GEMM_* code)."""
     name = {0: "k_gemm_tc", 1: "k_fdm_plane", 6: "k_fdm_cluster<4>", 7: "k_fdm_cluster<2>",
-            8: "k_gemm_tc + k_gemm_cp"}.get(code, "k_gemm_cp" if code in (3, 4, 5) else "k_gemm")
-    return name + (" + k_fdm_y" if fused_y and code not in (0, 1, 6, 7, 8) else "")
+            8: "k_gemm_tc + k_gemm_cp", 9: "k_oz_split + k_gemm_oz"}.get(code, "k_gemm_cp" if code in (3, 4, 5) else "k_gemm")
+    return name + (" + k_fdm_y" if fused_y and code not in (0, 1, 6, 7, 8, 9) else "")
 
 
 # DRAM traffic per launch of a transform kernel, from one ncu capture of an unchanged kernel
@@ -496,7 +496,8 @@ def main():
                         "peak_source": "measured FP32 FFMA peak of this GPU"}
             else:
                 peak = mp["fp64_tflops"]
-                roof = {"bound": "alu", "kernel": transform_kernel(gemm_choice, fused_y) + " (FP64 SIMT transforms)",
+                kind = " (FP64 by digit products)" if gemm_choice == native.PF_GEMM_DIGITS else " (FP64 SIMT transforms)"
+                roof = {"bound": "alu", "kernel": transform_kernel(gemm_choice, fused_y) + kind,
                         "peak_source": "measured FP64 DFMA peak of this GPU"}
             traffic = TRANSFORM_DRAM_BYTES_PER_LAUNCH.get((args.workload, args.precision, gemm_choice, fused_y))
             roof.update({"achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
@@ -559,7 +560,8 @@ def main():
                                     6: "whole solve per plane on a 4-block cluster (SIMT, distributed shared memory)",
                                     7: "whole solve per plane on a 2-block cluster (SIMT, distributed shared memory)",
                                     8: "hybrid: psi, phi solves SIMT 64x64 cp.async, V, P, u tcgen05 3xTF32 with "
-                                       "4-slice accumulation groups"}.get(gemm_choice, f"SIMT {gemm_choice}x{gemm_choice} tiles")
+                                       "4-slice accumulation groups",
+                                    9: "exact products of 8-bit digits on the tensor cores"}.get(gemm_choice, f"SIMT {gemm_choice}x{gemm_choice} tiles")
                                    + (", y pair fused" if fused_y and gemm_choice not in (0, 1, 6, 7) else "")
                                    + (" (autotuned)" if args.variant is None else " (pinned)"),
                        "fft_pencils_per_block": fft_tile,

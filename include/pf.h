@@ -52,9 +52,9 @@ extern "C" {
 #define PF_BC_NEUMANN   1
 #define PF_BC_PATCHES   2   /* wall only: electrodes on parts of the wall (eq. 21), see pf_vbc */
 
-#define PF_FP64  0   /* every kernel in double precision; the eigenbasis GEMMs of planes of   */
-                     /* 28 to 480 nodes a side as exact products of 8-bit digits on the       */
-                     /* tensor cores, unless pf_set_variant pins a CUDA-core variant          */
+#define PF_FP64  0   /* every kernel in double precision; the eigenbasis GEMMs of planes whose */
+                     /* longer side has 28 to 480 nodes as exact products of 8-bit digits on   */
+                     /* the tensor cores (PF_GEMM_DIGITS), unless another variant is chosen    */
 #define PF_MIXED 1   /* node-wise kernels and FFT in FP32, eigenbasis GEMMs in 3xTF32 on   */
                      /* the tensor cores (FP32 accumulation); set-up, the initial-potential */
                      /* fixed point and reductions in FP64                                  */
@@ -264,6 +264,8 @@ int pf_profile_read(pf_handle *h, double *ms, long long *launches);
  *                    the whole solve of a mode plane on a cluster of 4 / 2 thread blocks that
  *                    exchange the plane through distributed shared memory (FP32 precisions;
  *                    n_x <= 128, n_y <= 128)
+ *   PF_GEMM_DIGITS   exact products of 8-bit digits on the tensor cores (PF_FP64 only; what an FP64 run
+ *                    whose longer plane side has 28 to 480 nodes starts with)
  * All give the same result up to rounding order; in FP64 the CUDA-core variants sum in the same
  * order and agree bit for bit. */
 #define PF_GEMM_TC 0
@@ -277,14 +279,13 @@ int pf_profile_read(pf_handle *h, double *ms, long long *launches);
 #define PF_GEMM_CLUSTER4 6
 #define PF_GEMM_CLUSTER2 7
 #define PF_GEMM_TC_HYBRID 8
+#define PF_GEMM_DIGITS 9
 
 /* Autotuner of a single run: time `steps` steady steps with each transform variant available to
  * the run (PF_GEMM_*), keep the fastest, then (unless a whole-plane variant won) whether the y transforms
  * run fused (one pass, eigenbasis in shared memory), then (3D) the z-transform tile of 4, 8, 16
  * or 32 pencils per block.  Each candidate is timed as the run executes its steady steps: graph
- * replays when the run has its own stream, eager launches on the legacy stream.  An FP64 run that
- * is on the digit-product transforms times them as well and stays on them when they are fastest;
- * choice then names the fastest CUDA-core variant, ms_per_step the run's time.  The run advances
+ * replays when the run has its own stream, eager launches on the legacy stream.  The run advances
  * by 16 (steps + 2) steps.  choice (nullable) receives gemm + 1000 * tile + 100000 * fused_y with
  * gemm a PF_GEMM_* code, tile the pencils per z-transform block (0: size heuristic, always 0 in
  * 2D) and fused_y 1 when the y pair runs fused; ms_per_step (nullable) the best time. */
@@ -295,8 +296,8 @@ int pf_autotune(pf_handle *h, int steps, int *choice, double *ms_per_step);
  * (0 separately; ignored by the whole-plane variants), tile the pencils per z-transform block (4, 8, 16,
  * 32) or 0 for the size heuristic.  Synchronises the run's stream and drops its captured
  * graphs.  PF_EINVAL (nothing changed) when a value is outside these sets or the run cannot use
- * the variant (PF_GEMM_TC outside PF_MIXED, the whole-plane variants in FP64 or on a plane too
- * large). */
+ * the variant (PF_GEMM_TC outside PF_MIXED, PF_GEMM_DIGITS in an FP64 run that does not start with it,
+ * the whole-plane variants in FP64 or on a plane too large). */
 int pf_set_variant(pf_handle *h, int gemm, int fuse_y, int tile);
 
 /* Accumulation of the 3xTF32 tensor-core transforms (the constant eigenbasis products of the

@@ -577,8 +577,9 @@ struct Engine {
     // ---- FP64 transforms by exact digit products on the tensor cores (pf_oz.cuh) -----------------
     static int oz_kpad(int k) { return pf::oz_kpad(k); }
     // Eight launches a solve of about 5 us at least against the SIMT transforms' three or four: measured
-    // per 2D step, 24 x 13 nodes 0.277 / 0.271 ms (digits / SIMT), 30 x 16 0.279 / 0.289, 48 x 25 0.310 /
-    // 0.384, 240 x 121 0.571 / 1.276
+    // per 2D step, digits / fastest SIMT variant, 30 x 16 nodes 0.265 / 0.266 ms, 32 x 17 0.276 / 0.276, 48 x 25
+    // 0.300 / 0.367, 105 x 43 0.354 / 0.611, 240 x 121 0.505 / 1.252, 480 x 241 0.958 / 2.857 (24 x 13, with seven
+    // digits: 0.277 / 0.271)
     // The FP64 engine that only finds a mixed run's initial potential keeps the FMA transforms: a last bit
     // of V^0 moves the FP32 rounding of every later step (P by 1e-5 after four steps).
     bool oz_pays() const {
@@ -1050,14 +1051,14 @@ struct Engine {
     bool gemm_available(int code) const {
         return ((code == 0 || code == 8) && !tcb.empty()) || (code == 1 && plane_fits()) || code == 32 ||
                code == 64 || (code >= 2 && code <= 5) || (code == 6 && cluster_fits(4)) ||
-               (code == 7 && cluster_fits(2));
+               (code == 7 && cluster_fits(2)) || (code == PF_GEMM_DIGITS && !ozb.empty());
     }
     // PF_GEMM_TC_HYBRID (8): the psi and phi solves (the natural-BC set) on the cp.async 64x64 SIMT
     // transforms, the others on the tensor cores with four K slices per accumulation group
     bool tc_hybrid = false;
     void set_gemm(int code) {
         use_tc = code == 0 || code == 8;
-        use_oz = false;
+        use_oz = code == PF_GEMM_DIGITS;
         tc_hybrid = code == 8;
         fuse_plane = code == 1;
         cluster = code == 6 ? 4 : code == 7 ? 2 : 0;
@@ -2158,14 +2159,10 @@ void autotune_engine(Engine<T> &E, int steps, int total, cudaEvent_t e0, cudaEve
         PF_CU(cudaEventElapsedTime(&ms, e0, e1));
         return (double)ms / steps;
     };
-    // a run on the FP64 digit-product transforms times them first: they have no code of their own, and
-    // stay when no variant beats them
-    const bool digits = E.use_oz;
     int taken = 0;
-    const double digits_ms = digits ? time_variant(taken) : INFINITY;
     // every variant this engine can run (PF_GEMM_* codes)
     std::vector<int> cands;
-    for (int code : {0, 8, 32, 64, 2, 3, 4, 5, 1, 6, 7})
+    for (int code : {0, 8, PF_GEMM_DIGITS, 32, 64, 2, 3, 4, 5, 1, 6, 7})
         if (E.gemm_available(code)) cands.push_back(code);
     int pick = cands[0];
     double best = INFINITY;
@@ -2175,10 +2172,6 @@ void autotune_engine(Engine<T> &E, int steps, int total, cudaEvent_t e0, cudaEve
         if (ms < best) { best = ms; pick = code; }
     }
     E.set_gemm(pick);
-    if (digits_ms < best) {
-        E.use_oz = true;
-        best = digits_ms;
-    }
     // the fused y pair against the two separate y transforms (the whole-plane solves have no y pair)
     if (!E.fuse_plane && !E.cluster && !E.use_oz) {
         E.fuse_y = !E.fuse_y;
@@ -2198,7 +2191,7 @@ void autotune_engine(Engine<T> &E, int steps, int total, cudaEvent_t e0, cudaEve
     }
     drop_graphs();
     for (; taken < total; ++taken) E.step(2);
-    if (choice) *choice = pick + 1000 * E.tp_override + ((E.fuse_y && !E.fuse_plane && !E.cluster) ? 100000 : 0);
+    if (choice) *choice = pick + 1000 * E.tp_override + ((E.fuse_y && !E.fuse_plane && !E.cluster && !E.use_oz) ? 100000 : 0);
     if (best_ms) *best_ms = best;
 }
 }  // namespace
@@ -2207,7 +2200,7 @@ extern "C" int pf_autotune(pf_handle *h, int steps, int *choice, double *ms_per_
     if (!h || steps < 1) return PF_EINVAL;
     try {
         if (h->nstep < 1) pf_step(h, 1);
-        int total = 16 * (steps + 2);   // at most 11 transform variants + the y pair + 4 tiles
+        int total = 16 * (steps + 2);   // at most 11 transform variants (FP32: 11, FP64: 7) + the y pair + 4 tiles
         cudaEvent_t e0, e1;
         PF_CU(cudaEventCreate(&e0));
         PF_CU(cudaEventCreate(&e1));
@@ -2686,15 +2679,12 @@ extern "C" int pf_batch_autotune(pf_batch *b, int steps, double *ms_out) {
             double best = INFINITY;
             for_engine(g, [&](auto &E) {
                 std::vector<int> cands;
-                for (int code : {0, 32, 64, 1, 6, 7})
+                for (int code : {0, PF_GEMM_DIGITS, 32, 64, 1, 6, 7})
                     if (E.gemm_available(code)) cands.push_back(code);
-                // the FP64 digit-product transforms (code -1 here) are timed too
-                if (E.use_oz) cands.push_back(-1);
                 int pick = cands[0];
                 int taken = 0;
                 for (int code : cands) {
-                    if (code < 0) E.use_oz = true;
-                    else E.set_gemm(code);
+                    E.set_gemm(code);
                     E.step(2);   // warm-up of this variant
                     PF_CU(cudaEventRecord(e0, E.st));
                     for (int s = 0; s < steps; ++s) E.step(2);
@@ -2705,8 +2695,7 @@ extern "C" int pf_batch_autotune(pf_batch *b, int steps, double *ms_out) {
                     PF_CU(cudaEventElapsedTime(&ms, e0, e1));
                     if (ms / steps < best) { best = ms / steps; pick = code; }
                 }
-                if (pick < 0) E.use_oz = true;
-                else E.set_gemm(pick);
+                E.set_gemm(pick);
                 for (; taken < total; ++taken) E.step(2);
             });
             if (ms_out) ms_out[gi] = best;
