@@ -544,31 +544,18 @@ struct Engine {
             raise_smem_limit((const void *)pf::k_gemm_tc, most);
         }
         if (sizeof(T) == 8 && oz_pays()) {
-            use_oz = true;
-            auto tr = [](const std::vector<double> &m, int n) {
-                std::vector<double> t((size_t)n * n);
-                for (int i = 0; i < n; ++i)
-                    for (int j = 0; j < n; ++j) t[(size_t)i * n + j] = m[(size_t)j * n + i];
-                return t;
-            };
-            add_oz(Sx, tr(s.Sx, nx), nx);
-            add_oz(SxT, s.Sx, nx);
-            for (int b = 0; b < 4; ++b) {
-                add_oz(Sy[b], tr(s.Sy[b], ny), ny);
-                add_oz(SyT[b], s.Sy[b], ny);
-            }
-            raise_smem_limit((const void *)pf::k_gemm_oz, pf::OZ_SMEM);
-            const long long most = (s.model == PF_MODEL_EQUILIBRIUM ? 1ll : d3 ? 3ll : 2ll) * nz;   // planes of a solve
-            ozdig = mk<__half>((size_t)pf::OZ_S * most * std::max((long long)ny * oz_kpad(nx), (long long)nx * oz_kpad(ny)));
-            ozE = mk<int>(most * std::max(nx, ny));
-            // reciprocals for the solves of the steady step (the others divide)
-            const int j = s.bdf == 2 ? 1 : 0;
-            add_rcp(PF_BCSET_V, shV);
-            add_rcp(PF_BCSET_NN, shPsi[j]);
-            add_rcp(PF_BCSET_NN, shPhi[j]);
-            if (s.model != PF_MODEL_EQUILIBRIUM) {
-                add_rcp(PF_BCSET_P, shP);
-                add_rcp(PF_BCSET_U, shU[j]);
+            const size_t before = allocs.size();
+            try {
+                build_oz(s);
+                use_oz = true;
+            } catch (const CudaError &e) {   // a run that fits without the digits' memory runs on the FMA transforms
+                if (e.code != cudaErrorMemoryAllocation) throw;
+                PF_CU(cudaStreamSynchronize(st));
+                for (; allocs.size() > before; allocs.pop_back()) cudaFree(allocs.back());
+                ozb.clear();
+                ozrcp.clear();
+                ozdig = nullptr;
+                ozE = nullptr;
             }
         }
         PF_CU(cudaStreamSynchronize(st));
@@ -585,6 +572,36 @@ struct Engine {
     bool oz_pays() const {
         return hs.precision == PF_FP64 && std::max(nx, ny) >= 28 && nx <= pf::OZ_MAXK && ny <= pf::OZ_MAXK &&
                tc_encode() != nullptr;
+    }
+    // digits of the eigenbases and of the A operands (16 B a value of the largest solve: of three velocity
+    // components in 3D, two in 2D, one field of the equilibrium system) and the reciprocals (in 3D 8 B a value and
+    // table, in 2D 16 B a node; five tables, three for the equilibrium system)
+    void build_oz(const HostSetup &s) {
+        auto tr = [](const std::vector<double> &m, int n) {
+            std::vector<double> t((size_t)n * n);
+            for (int i = 0; i < n; ++i)
+                for (int j = 0; j < n; ++j) t[(size_t)i * n + j] = m[(size_t)j * n + i];
+            return t;
+        };
+        add_oz(Sx, tr(s.Sx, nx), nx);
+        add_oz(SxT, s.Sx, nx);
+        for (int b = 0; b < 4; ++b) {
+            add_oz(Sy[b], tr(s.Sy[b], ny), ny);
+            add_oz(SyT[b], s.Sy[b], ny);
+        }
+        raise_smem_limit((const void *)pf::k_gemm_oz, pf::OZ_SMEM);
+        const long long most = (s.model == PF_MODEL_EQUILIBRIUM ? 1ll : d3 ? 3ll : 2ll) * nz;   // planes of a solve
+        ozdig = mk<__half>((size_t)pf::OZ_S * most * std::max((long long)ny * oz_kpad(nx), (long long)nx * oz_kpad(ny)));
+        ozE = mk<int>(most * std::max(nx, ny));
+        // reciprocals for the solves of the steady step (the others divide)
+        const int j = s.bdf == 2 ? 1 : 0;
+        add_rcp(PF_BCSET_V, shV);
+        add_rcp(PF_BCSET_NN, shPsi[j]);
+        add_rcp(PF_BCSET_NN, shPhi[j]);
+        if (s.model != PF_MODEL_EQUILIBRIUM) {
+            add_rcp(PF_BCSET_P, shP);
+            add_rcp(PF_BCSET_U, shU[j]);
+        }
     }
     // digits and exponents of Bt's rows (Bt n x n row-major: B's columns), balanced by the shifts of B's rows
     void add_oz(const T *key, const std::vector<double> &Bt, int n) {
