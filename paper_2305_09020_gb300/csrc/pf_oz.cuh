@@ -268,17 +268,18 @@ __device__ __forceinline__ void oz_split_row(const double *__restrict__ row, int
 template <int NI>
 __global__ void __launch_bounds__(256) k_oz_split(const double *__restrict__ A, int M, int K, int Kpad, const int *__restrict__ sh,
                                                   __half *__restrict__ dig, int *__restrict__ E, int R,
-                                                  const int *__restrict__ active, int amod) {
+                                                  const int *__restrict__ active, int amod, const int *__restrict__ skip_if) {
     const int m = blockIdx.x * 8 + (threadIdx.x >> 5);
     tc_pdl_enter();
-    if (m >= M) return;
+    if (m >= M || (skip_if && *skip_if)) return;
     if (active && !active[(m / R) % amod]) return;   // a frozen run's rows: their products are not used
     oz_split_row<NI>(A + (long long)m * K, 1, sh, 1, m, M, K, Kpad, dig, E, nullptr);
 }
 
-// launch of k_oz_split for the M rows of A (K <= OZ_MAXK values each); pdl: as a programmatic dependent launch
+// launch of k_oz_split for the M rows of A (K <= OZ_MAXK values each); pdl: as a programmatic dependent launch;
+// skip_if: as OzArgs
 inline void oz_split(const double *A, int M, int K, const int *sh, __half *dig, int *E, int R, const int *active, int amod,
-                     cudaStream_t st, bool pdl = false) {
+                     cudaStream_t st, bool pdl = false, const int *skip_if = nullptr) {
     const int Kpad = oz_kpad(K);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((M + 7) / 8));
@@ -289,8 +290,8 @@ inline void oz_split(const double *A, int M, int K, const int *sh, __half *dig, 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
-    auto go = [&](void (*k)(const double *, int, int, int, const int *, __half *, int *, int, const int *, int)) {
-        cudaLaunchKernelEx(&cfg, k, A, M, K, Kpad, sh, dig, E, R, active, amod);   // errors: the caller's cudaGetLastError
+    auto go = [&](void (*k)(const double *, int, int, int, const int *, __half *, int *, int, const int *, int, const int *)) {
+        cudaLaunchKernelEx(&cfg, k, A, M, K, Kpad, sh, dig, E, R, active, amod, skip_if);   // errors: the caller's cudaGetLastError
     };
     switch ((Kpad + 63) / 64) {
         case 1: go(k_oz_split<1>); break;

@@ -111,7 +111,7 @@ int launch_digits(Digits *D, int sms, const double *A, int b, double *C, long lo
         pf_internal_set_error("cuTensorMapEncodeTiled failed");
         return PF_ECUDA;
     }
-    pf::oz_split(A, (int)rows, n, D->sh[b], D->a, D->E, R, nullptr, 1, st);
+    pf::oz_split(A, (int)rows, n, D->sh[b], D->a, D->E, R, nullptr, 1, st, false, &D->sparse);
     pf::k_gemm_oz<<<(unsigned)(a.nunits < sms ? a.nunits : sms), pf::OZ_THREADS, smem, st>>>(ma, mb, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
