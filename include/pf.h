@@ -448,8 +448,11 @@ void pf_no_destroy(pf_no *h);
  *
  * Its two intermediate buffers live in one file-scope device array of
  * 2 * PF_STATIC_MAX_VALUES doubles (16 MiB) that every GPU loading this library holds
- * until exit, the operands' digits of its tensor-core transforms in a second one (42 MB; planes of 16
- * to 480 nodes a side take those, a wait that gives up there leaves NaN in out).
+ * until exit, the operands' digits of its tensor-core transforms in a second one (49 MB; planes of 16
+ * to 480 nodes a side take those, a wait that gives up there leaves NaN in out; where an eigenbasis has
+ * zeros inside rows and columns that are not zero, as an interior Dirichlet node makes them, the CUDA-core
+ * kernels run).  Right-hand side values at constrained nodes (zero rows of Sx, Sy) do not enter unless they
+ * are not finite.
  * nx*ny*nplanes > PF_STATIC_MAX_VALUES returns PF_EINVAL (message in
  * pf_last_error(NULL)).  The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current and keeps it for the life of the process;

@@ -2471,7 +2471,8 @@ __global__ void k_energy(Geo<T> G, EnergyConst c, const T *__restrict__ phi, con
 
 // up to ten fields of n values as FP64 blocks in mapped (pinned) host memory, zeros for a null source: the
 // conversion and the way over the link in one launch for all fields (a conversion into scratch and a copy
-// per field: two launches each, and the link idle during the conversions)
+// per field: two launches each, and the link idle during the conversions).  Its blocks hold SMs while the link
+// is busy: other streams' kernels share them for that long, where copies would have left them free.
 template <typename T>
 struct FieldsOut {
     const T *src[10];

@@ -20,14 +20,13 @@
 // which is exact but for v_7; |acc| < 2^62 for K < 512.  The result is rounded to double once.
 //
 // The error is relative to the largest balanced entries, an FMA chain's to the sum of the terms' sizes.
-// Balanced, the largest entry of A meets an entry of its own size in B's row, so that the row of C holds a value
-// as large as that product, and eight digits leave 2^-61 of it where a chain leaves 2^-53 per term: no plane, row
-// or column of a solve is further off than with the chains (tests: even, cosine and geometric meshes to a ratio
+// Balanced, the largest entry of A meets the largest entry of B's row, so that one term of the row of C is
+// as large as their product, and eight digits leave 2^-61 of it where a chain leaves 2^-53 per term: no plane, row
+// or column of the solves tested is further off than with the chains (even, cosine and geometric meshes to a ratio
 // of 4^10 in size, values of 1e200 at constrained nodes).  Measured against extended precision, 105 x 43
 // nodes on a cosine mesh, plane / worst row / worst column: chains 8.4e-16 / 1.3e-15 / 2.9e-15, seven digits
 // without the balance 1.1e-15 / 6.1e-14 / 5.7e-15 (and no digit left for a value of 1e16 at a constrained node),
-// seven with it 6e-16 / 1.6e-14 / 4e-15, these 1.2e-16 /
-// 2.0e-16 / 3.0e-16.
+// seven with it 6e-16 / 1.6e-14 / 4e-15 (emulated), these 1.2e-16 / 2.0e-16 / 3.0e-16.
 // What cannot be balanced per k is a basis of uncoupled pieces (zeros inside rows and columns that are not
 // zero): entries of one piece would take digits from another.  The allocation-free solve, whose bases are the
 // caller's, finds those on the device and takes the FMA kernels (pf_static.cu); a run's own have none.

@@ -123,9 +123,9 @@ int launch_digits(Digits *D, int sms, const double *A, int b, double *C, long lo
 
 // The tensor-core transforms take ten launches (the eigenbases are split anew in each call: they
 // are the caller's) and the four of the FMA kernels, which return at once unless a basis falls into uncoupled
-// pieces, and are the faster ones from the smallest planes measured on: 32 x 17 nodes,
-// one plane 149 -> 80 us; 128 x 65, one plane 451 -> 107 us, 64 planes 607 -> 133 us; 240 x 121, 30 planes
-// 1547 -> 170 us.
+// pieces, and are the faster ones from the smallest planes measured on (FMA kernels alone / these): 16 x 17 nodes,
+// one plane 124 / 95 us; 32 x 17 158 / 101; 128 x 65, one plane 462 / 123, 64 planes 620 / 160; 240 x 145, 30 planes
+// 1977 / 218.  A basis of uncoupled pieces pays 35 to 50 us for the launches that return at once.
 bool digits_fit(int nx, int ny, long long total) {
     if (nx < DIG_MIN || ny < DIG_MIN || nx > pf::OZ_MAXK || ny > pf::OZ_MAXK || pf::tc_encode() == nullptr) return false;
     const long long P = total / ((long long)nx * ny);

@@ -268,8 +268,11 @@ __device__ __forceinline__ void tmem_add(uint32_t taddr, int hbn, float *acc) {
 // acc[j] /= lam[j] + lr for 32 columns whose sums the host has found to lie in [1e-15, 1e15]: a
 // division operator per column costs a branch each (operands out of its fast path's range) that keeps
 // the next one from starting, 16,000 cycles for a tile's 64.  Here the quotient is the product with the
-// approximate reciprocal plus one residual correction (Markstein), q += (x - q d) r, which leaves less
-// than one unit in the last place.  lam is 16-byte aligned and padded to whole store rounds.
+// approximate reciprocal plus one residual correction (Markstein), q += (x - q d) r.  The reciprocal is within
+// two units in its last place, so that the sum before its one rounding is the quotient to 2^-44: the result is
+// the division operator's but for ties within 1e-6 of a unit (none to 9 of 20 million quotients, emulated
+// with the reciprocal 0, 1 and 2 units off).  Only values near the subnormal range, whose residual underflows, keep
+// the first product's error.  lam is 16-byte aligned and padded to whole store rounds.
 __device__ __forceinline__ void div_cols(float *acc, const float *lam, float lr) {
 #pragma unroll
     for (int j = 0; j < TC_OUT; j += 4) {
